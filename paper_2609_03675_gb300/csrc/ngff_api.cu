@@ -309,7 +309,13 @@ cudaError_t launch_first_stage(cofie_ngff* h, const SegTable& segs, cudaStream_t
   ha.chunks_per_frame = (ha.groups_per_frame + hist_chunk_groups() - 1) / hist_chunk_groups();
   ha.timeout_ns = kTimeoutNs;
   if (cells) {
-    if (!fast) return launch_features(segs, h->fa, h->lc, h->d_hist, h->fw, st);
+    const bool dhash = h->p.signal == COFIE_SIGNAL_DHASH;
+    uint32_t* cells_out = dhash ? h->d_cells : h->d_hist;
+    if (!fast) {
+      cudaError_t e = launch_cells_any(segs, h->fa, h->lc, cells_out, h->num_sms, st, pdl);
+      if (e == cudaSuccess && dhash) e = launch_dhash_finish(h->d_cells, segs.rows, h->fa, h->d_hist, st, true);
+      return e;
+    }
     ha.width = h->p.width;
     ha.height = h->p.height;
     ha.grid_h = h->fa.grid_h;
@@ -321,8 +327,7 @@ cudaError_t launch_first_stage(cofie_ngff* h, const SegTable& segs, cudaStream_t
     ha.wide = (h->p.width / h->fa.grid_w >= 16 && h->m_gw) ? 1u : 0u;
     const uint64_t chunks = static_cast<uint64_t>(segs.rows) * ha.chunks_per_frame;
     const int grid = static_cast<int>(chunks < static_cast<uint64_t>(h->cells_grid) ? chunks : h->cells_grid);
-    const bool dhash = h->p.signal == COFIE_SIGNAL_DHASH;
-    cudaError_t e = launch_cells_fast(segs, ha, h->lc, dhash ? h->d_cells : h->d_hist, h->d_err, grid, st, pdl);
+    cudaError_t e = launch_cells_fast(segs, ha, h->lc, cells_out, h->d_err, grid, st, pdl);
     if (e == cudaSuccess && dhash) e = launch_dhash_finish(h->d_cells, segs.rows, h->fa, h->d_hist, st, true);
     return e;
   }
@@ -688,7 +693,8 @@ int cofie_ngff_create(const cofie_ngff_params* p, cofie_ngff_t** out) {
     fa.npix = h->npix;
     fa.grid_h = p->signal == COFIE_SIGNAL_LOWRES ? 16 : 8;
     fa.grid_w = p->signal == COFIE_SIGNAL_LOWRES ? 16 : 9;
-    fa.kind = p->signal;
+    fa.m_col = static_cast<uint32_t>(
+        std::min<uint64_t>((static_cast<uint64_t>(fa.grid_w) << 32) / p->width, 0xffffffffull));
     for (uint32_t y = 0; y < p->height; ++y) fa.row_h[y * fa.grid_h / p->height] += 1;
     for (uint32_t x = 0; x < p->width; ++x) fa.col_w[x * fa.grid_w / p->width] += 1;
   }

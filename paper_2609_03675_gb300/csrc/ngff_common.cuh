@@ -195,8 +195,9 @@ struct FeatArgs {
   uint64_t frame_bytes;
   uint32_t width, height, npix;
   uint32_t grid_h, grid_w;    // cell rows, cell columns
-  uint32_t kind;              // 1: low-res (writes the cell sums), 2: dHash (writes 64 bits)
   uint32_t use_magic;         // Y = umulhi(v, magic_y) (host-verified), else v / den
+  uint32_t m_col;             // floor(2^32 grid_w / width), at most 2^32 - 1
+  uint32_t slice_groups, slices;  // a launch's 16-pixel groups per CTA, and CTAs per frame
   uint32_t row_h[16], col_w[16];  // pixels per cell row / cell column
 };
 
@@ -245,8 +246,8 @@ uint32_t select_walk_max_frames();
 uint32_t select_walk_max_lmax();
 cudaError_t launch_select_walk(const SegTable& segs, const SelectArgs& a, uint32_t* hist, uint32_t* ring,
                                StreamState* state, cudaStream_t st, bool pdl = false);
-cudaError_t launch_features(const SegTable& segs, const FeatArgs& fa, const LumaConsts& lc, uint32_t* feat, uint32_t fw,
-                            cudaStream_t st);
+cudaError_t launch_cells_any(const SegTable& segs, const FeatArgs& fa, const LumaConsts& lc, uint32_t* cells,
+                             int num_sms, cudaStream_t st, bool pdl = false);
 int cells_blocks_per_sm();
 cudaError_t launch_cells_fast(const SegTable& segs, const HistArgs& a, const LumaConsts& lc, uint32_t* cells,
                               uint32_t* err, int grid, cudaStream_t st, bool pdl = false);

@@ -2,87 +2,160 @@
 // kernel does not apply, the dHash bits from cell sums, the bounded-wait
 // probe of the failure path, and the bin check over arbitrary pixels. They
 // share K1's grayscale and bin functions (ngff_device.cuh).
+#include <algorithm>
+
 #include "ngff_device.cuh"
 
 namespace cofie {
 namespace {
 
-// The spatial signals (low-res difference, dHash) where the TMA kernel does
-// not apply (width not a multiple of 16, unaligned frames, or no verified
-// multiply-high for the grayscale division): one CTA per frame sums the
-// grayscale of each cell of a grid_h x grid_w grid in shared memory. Fast path
-// (width a multiple of 16, aligned frames): 16-pixel groups, the same dp2a
-// luma as the histogram kernel, runs of pixels of one cell added in registers
-// and flushed with one shared atomic per run. Then low-res writes the cell
-// sums, dHash the 64 bits [mean(r, c) > mean(r, c + 1)] compared exactly by
-// cross-multiplying sums and pixel counts.
-constexpr int kFeatThreads = 512;
+// The spatial signals (low-res difference, dHash) where the bulk-copy kernel
+// does not apply: a width that is no multiple of 16, frames that do not start
+// on a 16-byte boundary, or no verified multiply-high for the grayscale
+// division. CTA x of the grid sums one slice of one frame's pixels by cell.
+// As in the generic histogram kernel a frame's pixels split into a prologue
+// of fewer than 16 pixels, whole 16-pixel groups that start on a 16-byte
+// boundary (three 128-bit loads, two dp2a per pixel) and an epilogue of fewer
+// than 16. Groups take no notice of where image rows end: in row-major order
+// the cell columns of a row, and the first column of the row below, are
+// consecutive runs of pixels, so with columns of at least 16 pixels (kWide) a
+// group meets at most one boundary, the end of a cell column or of the row,
+// and is split there as the bulk-copy kernel splits its groups; narrower
+// columns take a loop over the pixels. A thread's next group is
+// 16 kAnyThreads pixels on, so its row and column advance by additions, and
+// its cell row by comparison with the row where the next one starts.
+//
+// Bound by memory latency: about 150 issue slots per 48 bytes, so the more
+// warps there are to cover a load, the nearer the kernel comes to DRAM's rate.
+// Hence registers for six CTAs per SM and sums formed as the pixels are
+// decoded, without arrays of prefix sums (four CTAs: 5 % slower over 600
+// frames of 854x480; eight, which spill: 7 %). Lanes of a warp hold
+// neighbouring groups, of which several fall in one cell; each cell is kept
+// kCellCopies times, a lane adding to copy lane mod kCellCopies (4 and 16
+// copies measured the same). Those 600 frames (738 MB) take 0.12 ms, 6.2 TB/s;
+// the kernel this one replaced, a CTA per frame with byte loads and a division
+// per pixel, took 0.79 ms.
+constexpr int kAnyThreads = 256;
+constexpr uint32_t kAnyGroups = 2048;    // 16-pixel groups per CTA, fewer for small launches
+constexpr uint32_t kAnyGroupsMin = 256;
+constexpr uint32_t kCellCopies = 8;
 
-__global__ void __launch_bounds__(kFeatThreads) features_kernel(SegTable segs, FeatArgs fa, LumaConsts L,
-                                                                uint32_t* __restrict__ feat, uint32_t fw) {
-  __shared__ uint32_t cell[256];
+template <bool kDiv, bool kWide>
+__global__ void __launch_bounds__(kAnyThreads, 6) cells_any_kernel(SegTable segs, FeatArgs fa, LumaConsts L,
+                                                                uint32_t* __restrict__ cells) {
+  __shared__ __align__(16) uint32_t cell[256 * kCellCopies];
+  __shared__ uint32_t colstart[17];
   pdl_trigger();
-  const uint32_t row = blockIdx.x, tid = threadIdx.x;
+  const uint32_t tid = threadIdx.x, lane = tid & 31;
+  const uint32_t row = blockIdx.x / fa.slices, slice = blockIdx.x - row * fa.slices;
   uint32_t seg = 0;
   while (seg + 1 < segs.count && row >= segs.s[seg + 1].row0) ++seg;
   const uint8_t* frame = segs.s[seg].frames + static_cast<uint64_t>(row - segs.s[seg].row0) * fa.frame_bytes;
-  const uint32_t gh = fa.grid_h, gw = fa.grid_w, W = fa.width, H = fa.height;
-  for (uint32_t i = tid; i < gh * gw; i += kFeatThreads) cell[i] = 0;
+  const uint32_t gh = fa.grid_h, gw = fa.grid_w, W = fa.width, H = fa.height, n_cells = gh * gw;
+  const uint32_t gh_shift = 31 - __clz(gh);  // 8 or 16 cell rows
+  for (uint32_t i = tid; i < n_cells * kCellCopies; i += kAnyThreads) cell[i] = 0;
+  if (tid <= gw) colstart[tid] = static_cast<uint32_t>((static_cast<uint64_t>(tid) * W + gw - 1) / gw);
+  pdl_wait();  // no frame is read and no cell written before the kernel before this one has completed
   __syncthreads();
-  const bool fast = (W % 16 == 0) && (reinterpret_cast<uintptr_t>(frame) % 16 == 0) && (fa.frame_bytes % 16 == 0);
-  if (fast) {
-    const uint32_t gpr = W / 16, groups = fa.npix / 16;
-    for (uint32_t g = tid; g < groups; g += kFeatThreads) {
-      const uint32_t y = g / gpr, x0 = (g - y * gpr) * 16;
-      const uint32_t cy = y * gh / H;
-      const uint4* p4 = reinterpret_cast<const uint4*>(frame + static_cast<uint64_t>(g) * 48);
-      const uint4 a = p4[0], b = p4[1], c = p4[2];
-      uint32_t v[16];
-      luma4(a.x, a.y, a.z, L, v[0], v[1], v[2], v[3]);
-      luma4(a.w, b.x, b.y, L, v[4], v[5], v[6], v[7]);
-      luma4(b.z, b.w, c.x, L, v[8], v[9], v[10], v[11]);
-      luma4(c.y, c.z, c.w, L, v[12], v[13], v[14], v[15]);
-      uint32_t cx = x0 * gw / W;
-      uint32_t next = ((cx + 1) * W + gw - 1) / gw;  // first x of the next cell column
-      uint32_t acc = 0;
+
+  const auto floor_y = [&](uint32_t v) { return kDiv ? v / L.den : __umulhi(v, L.magic_y); };
+  const auto add = [&](uint32_t c, uint32_t sum) {
+    if (COFIE_BOUND(c < n_cells)) atomicAdd(&cell[c * kCellCopies + (lane & (kCellCopies - 1))], sum);
+  };
+  // first image row of the cell row after crow
+  const auto next_cell_row = [&](uint32_t crow) { return ((crow + 1) * H + gh - 1) >> gh_shift; };
+
+  // first 16-byte aligned pixel: 3 p = -(frame mod 16) mod 16, and 3 * 11 = 1 mod 16
+  const uint32_t mis = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(frame) & 15u);
+  const uint32_t p_a = min(((16u - mis) * 11u) & 15u, fa.npix);
+  const uint32_t G = (fa.npix - p_a) / 16;
+  const uint32_t g0 = slice * fa.slice_groups, g1 = min(g0 + fa.slice_groups, G);
+  const uint8_t* base = frame + 3ull * p_a;
+  if (g0 + tid < g1) {
+    const uint32_t q = p_a + 16 * (g0 + tid);
+    const uint32_t dr = 16 * kAnyThreads / W, dx = 16 * kAnyThreads - dr * W;
+    uint32_t r = q / W, x = q - r * W;
+    uint32_t crow = r * gh / H, row_end = next_cell_row(crow);
+#pragma unroll 1
+    for (uint32_t g = g0 + tid; g < g1; g += kAnyThreads) {
+      const uint4* p = reinterpret_cast<const uint4*>(base + 48ull * g);
+      const uint4 a = __ldcs(p), b = __ldcs(p + 1), c = __ldcs(p + 2);
+      // cell column of x: m_col is below 2^32 gw / W by at most 1, so the
+      // estimate is the column or one less
+      uint32_t cx = __umulhi(x, fa.m_col);
+      cx += x >= colstart[cx + 1];
+      const uint32_t c0 = crow * gw + cx;
+      const uint32_t w[12] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y, c.z, c.w};
+      if (kWide) {
+        const uint32_t s = min(colstart[cx + 1] - x, 16u);  // pixels of the group before the boundary
+        uint32_t lo = 0, sum = 0;
 #pragma unroll
-      for (uint32_t i = 0; i < 16; ++i) {
-        const uint32_t yv = fa.use_magic ? __umulhi(v[i], L.magic_y) : v[i] / L.den;
-        if (x0 + i >= next) {
-          if (COFIE_BOUND(cy * gw + cx < gh * gw)) atomicAdd(&cell[cy * gw + cx], acc);
-          acc = 0;
-          ++cx;
-          next = ((cx + 1) * W + gw - 1) / gw;
+        for (uint32_t k = 0; k < 4; ++k) {
+          uint32_t v[4];
+          luma4(w[3 * k], w[3 * k + 1], w[3 * k + 2], L, v[0], v[1], v[2], v[3]);
+#pragma unroll
+          for (uint32_t i = 0; i < 4; ++i) {
+            const uint32_t y = floor_y(v[i]);
+            sum += y;
+            if (4 * k + i < s) lo += y;
+          }
         }
-        acc += yv;
+        add(c0, lo);
+        // past the boundary: the next column, or the first one of the row below
+        if (s < 16) add(cx + 1 < gw || r + 1 >= row_end ? c0 + 1 : crow * gw, sum - lo);
+      } else {
+        uint32_t acc = 0, ci = c0, xx = x, rr = r, cc = cx, cr = crow, end = row_end, nx = colstart[cx + 1];
+#pragma unroll
+        for (uint32_t k = 0; k < 4; ++k) {
+          uint32_t v[4];
+          luma4(w[3 * k], w[3 * k + 1], w[3 * k + 2], L, v[0], v[1], v[2], v[3]);
+#pragma unroll
+          for (uint32_t i = 0; i < 4; ++i, ++xx) {
+            if (xx == nx) {
+              add(ci, acc);
+              acc = 0;
+              if (++cc == gw) {
+                cc = xx = 0;
+                if (++rr >= end) end = next_cell_row(++cr);
+              }
+              ci = cr * gw + cc;
+              nx = colstart[cc + 1];
+            }
+            acc += floor_y(v[i]);
+          }
+        }
+        add(ci, acc);
       }
-      if (COFIE_BOUND(cy * gw + cx < gh * gw)) atomicAdd(&cell[cy * gw + cx], acc);
-    }
-  } else {
-    for (uint32_t p = tid; p < fa.npix; p += kFeatThreads) {
-      const uint8_t* px = frame + 3ull * p;
-      const uint32_t yv = (L.w[0] * px[0] + L.w[1] * px[1] + L.w[2] * px[2] + L.half) / L.den;
-      const uint32_t y = p / W, x = p - y * W;
-      const uint32_t ci = (y * gh / H) * gw + x * gw / W;
-      if (COFIE_BOUND(ci < gh * gw)) atomicAdd(&cell[ci], yv);
+      if (g + kAnyThreads < g1) {
+        x += dx;
+        r += dr;
+        if (x >= W) {
+          x -= W;
+          ++r;
+        }
+        while (r >= row_end) row_end = next_cell_row(++crow);
+      }
     }
   }
+  // the ragged edges: prologue (first slice of the frame) and epilogue (last)
+  const auto scalar = [&](uint32_t q) {
+    const uint8_t* px = frame + 3ull * q;
+    const uint32_t yv = (L.w[0] * px[0] + L.w[1] * px[1] + L.w[2] * px[2] + L.half) / L.den;
+    const uint32_t y = q / W, x = q - y * W;
+    add((y * gh / H) * gw + x * gw / W, yv);
+  };
+  if (slice == 0 && tid < p_a) scalar(tid);
+  if (slice == fa.slices - 1 && p_a + 16 * G + tid < fa.npix) scalar(p_a + 16 * G + tid);
   __syncthreads();
-  uint32_t* out = feat + static_cast<uint64_t>(row) * fw;
-  if (fa.kind == 1) {
-    for (uint32_t i = tid; i < gh * gw; i += kFeatThreads) out[i] = cell[i];
-  } else if (tid < 64) {  // warps 0 and 1: bit (r, c) of the 8 x 8 hash
-    const uint32_t r = tid / 8, c = tid % 8;
-    const uint64_t sa = cell[r * gw + c], sb = cell[r * gw + c + 1];
-    const uint64_t na = static_cast<uint64_t>(fa.row_h[r]) * fa.col_w[c];
-    const uint64_t nb = static_cast<uint64_t>(fa.row_h[r]) * fa.col_w[c + 1];
-    const uint32_t word = __ballot_sync(0xffffffffu, sa * nb > sb * na);
-    if ((tid & 31) == 0) out[tid >> 5] = word;
+  for (uint32_t i = tid; i < n_cells; i += kAnyThreads) {
+    const uint4 u = reinterpret_cast<const uint4*>(cell)[2 * i], w = reinterpret_cast<const uint4*>(cell)[2 * i + 1];
+    const uint32_t sum = u.x + u.y + u.z + u.w + w.x + w.y + w.z + w.w;
+    if (sum && COFIE_BOUND(row < segs.rows)) atomicAdd(cells + static_cast<uint64_t>(row) * n_cells + i, sum);
   }
 }
 
-// dHash from the 8 x 9 cell sums the fast kernel accumulated (row-major, 72
-// per frame): bit (r, c) = [S(r, c) n(r, c + 1) > S(r, c + 1) n(r, c)], the
+// dHash from the 8 x 9 cell sums the kernel before it accumulated (row-major,
+// 72 per frame): bit (r, c) = [S(r, c) n(r, c + 1) > S(r, c + 1) n(r, c)], the
 // comparison of the two cell means without division. The cell row is zeroed
 // for the next push once read.
 __global__ void __launch_bounds__(96) dhash_finish_kernel(uint32_t* __restrict__ cells, FeatArgs fa,
@@ -144,10 +217,28 @@ cudaError_t launch_dhash_finish(uint32_t* cells, uint32_t rows, const FeatArgs& 
   return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
-cudaError_t launch_features(const SegTable& segs, const FeatArgs& fa, const LumaConsts& lc, uint32_t* feat, uint32_t fw,
-                            cudaStream_t st) {
-  features_kernel<<<segs.rows, kFeatThreads, 0, st>>>(segs, fa, lc, feat, fw);
-  return cudaGetLastError();
+cudaError_t launch_cells_any(const SegTable& segs, const FeatArgs& fa, const LumaConsts& lc, uint32_t* cells,
+                             int num_sms, cudaStream_t st, bool pdl) {
+  FeatArgs f = fa;
+  const uint32_t groups = std::max(1u, fa.npix / 16);  // at least the whole groups, whatever the alignment
+  const auto slices = [&](uint32_t per) { return (groups + per - 1) / per; };
+  f.slice_groups = kAnyGroups;  // smaller slices until the grid has four CTAs for every SM
+  while (f.slice_groups > kAnyGroupsMin && static_cast<uint64_t>(slices(f.slice_groups)) * segs.rows < 4ull * num_sms)
+    f.slice_groups /= 2;
+  f.slices = slices(f.slice_groups);
+  f.slice_groups = ((groups + f.slices - 1) / f.slices + kAnyThreads - 1) / kAnyThreads * kAnyThreads;  // even slices
+  f.slices = slices(f.slice_groups);
+  const uint64_t ctas = static_cast<uint64_t>(f.slices) * segs.rows;
+  if (ctas > 0x7fffffffull) return cudaErrorInvalidConfiguration;
+  const bool wide = fa.width / fa.grid_w >= 16;
+  // a programmatic dependent only while its CTAs leave room on the SMs that
+  // the kernel before it still holds (as the generic histogram kernel)
+  pdl = pdl && ctas <= 4ull * num_sms;
+  const auto kernel = fa.use_magic ? (wide ? cells_any_kernel<false, true> : cells_any_kernel<false, false>)
+                                   : (wide ? cells_any_kernel<true, true> : cells_any_kernel<true, false>);
+  const cudaError_t e = launch_dependent(pdl, kernel, dim3(static_cast<uint32_t>(ctas)), dim3(kAnyThreads), 0, st, segs,
+                                         f, lc, cells);
+  return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
 cudaError_t launch_wait_probe(uint64_t timeout_ns, uint32_t* err, cudaStream_t st) {

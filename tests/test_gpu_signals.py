@@ -171,6 +171,38 @@ def test_signal_state_and_shards(kind):
     assert m.shape[0] == L
 
 
+# The kernel for frames that the bulk-copy kernel does not take: cell columns
+# on both sides of 16 pixels, groups that cross the end of an image row, rows
+# shorter than a group and longer than a thread's step, one slice and several
+# with a short last one, frames that start on any byte of 16.
+ANY_SHAPES = [(9, 8), (16, 16), (17, 31), (143, 9), (145, 24), (255, 40), (257, 33), (854, 60), (4097, 17), (5003, 16),
+              (1366, 48), (19, 2000)]
+
+
+@pytest.mark.parametrize("kind", [SO.LOWRES, SO.DHASH])
+@pytest.mark.parametrize("shape", ANY_SHAPES)
+def test_signal_any_width_and_alignment(kind, shape):
+    from paper_2609_03675_gb300 import NGFF
+    W, H = shape
+    if kind == SO.LOWRES and min(W, H) < 16:
+        pytest.skip("low-res needs 16 x 16")
+    rng = np.random.default_rng(W * 31 + H + kind)
+    fr = rng.integers(0, 256, (5, H, W, 3), dtype=np.uint8)
+    fr[3], fr[4] = 255, rng.integers(0, 2, (H, W, 3)) * 255
+    feats = np.stack([SO.features(x, O.Params(W, H), kind) for x in fr])
+    f = NGFF(W, H, signal=kind)
+    for offset in range(0, 16, 1 if W * H < 20000 else 5):
+        raw = torch.empty(fr.size + 16, dtype=torch.uint8, device="cuda")
+        part = raw[offset:offset + fr.size]
+        part.copy_(torch.from_numpy(fr.reshape(-1)))
+        f.reset()
+        _, _, h = f.push(part.view(fr.shape), return_hist=True)
+        got = h.cpu().numpy().view(np.uint32)
+        got = got.astype(np.int64) if kind == SO.LOWRES else _unpack(got)
+        assert np.array_equal(got, feats), f"offset {offset}"
+    f.status()
+
+
 @pytest.mark.parametrize("kind", [SO.LOWRES, SO.DHASH])
 def test_signal_unaligned_frames_and_plain_division(kind):
     """Frames at an odd address (the per-frame byte path) and a grayscale
