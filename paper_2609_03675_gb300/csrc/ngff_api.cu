@@ -69,6 +69,7 @@ struct cofie_ngff {
   int bin_path = -1;  // kBinFast, kBinTwoStep, or -1 (generic kernel only)
   bool size_fast = false;
   int hist_grid = 0;
+  int hist_stages = 0;   // K1's ring stages
   uint64_t generic_wave = 0;  // CTAs of the generic kernel resident at once (0: never chosen over K1)
   int cells_grid = 0;    // the TMA kernel's grid for the spatial signals (0: not usable)
   unsigned long long x_tau = 0, x_cut = 0, x_grad = 0;  // integer forms of the fp32 decisions
@@ -356,7 +357,7 @@ cudaError_t launch_first_stage(cofie_ngff* h, const SegTable& segs, cudaStream_t
   if (fast) {
     const uint64_t chunks = static_cast<uint64_t>(segs.rows) * ha.chunks_per_frame;
     const int grid = static_cast<int>(chunks < static_cast<uint64_t>(h->hist_grid) ? chunks : h->hist_grid);
-    return launch_hist_fast(segs, ha, h->lc, h->bin_path, h->d_hist, h->d_err, grid, st, pdl);
+    return launch_hist_fast(segs, ha, h->lc, h->bin_path, h->hist_stages, h->d_hist, h->d_err, grid, st, pdl);
   }
   return launch_hist_generic(segs, ha, h->lc, h->bin_path, h->d_hist, st);
 }
@@ -772,7 +773,7 @@ int cofie_ngff_create(const cofie_ngff_params* p, cofie_ngff_t** out) {
   }
   if (e == cudaSuccess && p->l_max > 0) e = scan_prepare(h->mask_words, p->l_max);
   if (e == cudaSuccess && h->bin_path >= 0) {
-    const int per_sm = hist_blocks_per_sm(h->bin_path, p->bins);
+    const int per_sm = hist_blocks_per_sm(h->bin_path, p->bins, &h->hist_stages);
     if (per_sm <= 0) e = cudaGetLastError() != cudaSuccess ? cudaErrorInvalidConfiguration : cudaErrorInvalidValue;
     h->hist_grid = h->num_sms * (per_sm > 0 ? per_sm : 1);
     const int gen_per_sm = hist_generic_blocks_per_sm(h->bin_path, p->bins);

@@ -221,10 +221,10 @@ inline bool injected_alloc_failure() {
 }
 
 // Launchers (stream-ordered; return the launch error).
-int hist_blocks_per_sm(int bin_path, uint32_t bins);
+// K1's resident CTAs per SM (-1 on error) and the ring stages that give them
+int hist_blocks_per_sm(int bin_path, uint32_t bins, int* stages);
 uint32_t hist_chunk_groups();
-size_t hist_smem_bytes(uint32_t bins);
-cudaError_t launch_hist_fast(const SegTable& segs, const HistArgs& a, const LumaConsts& lc, int bin_path,
+cudaError_t launch_hist_fast(const SegTable& segs, const HistArgs& a, const LumaConsts& lc, int bin_path, int stages,
                              uint32_t* hist, uint32_t* err, int grid, cudaStream_t st, bool pdl = false);
 // The generic kernel over CTAs of slice_groups 16-pixel groups (0: the
 // default 2048); with pdl a programmatic dependent of the kernel before it.

@@ -68,9 +68,14 @@ struct Shape {
   static constexpr int warps = kBin == kCells ? kCellWarps : kConsumerWarps;
   static constexpr int consumers = warps * 32;
   static constexpr int threads = consumers + 32;
-  static constexpr int stages = kBin == kCells ? COFIE_CELL_STAGES : COFIE_K1_STAGES;
 };
 constexpr int kStages = COFIE_K1_STAGES;
+// With many bins the counters (128 bytes a bin) and a ring of kStages no
+// longer fit an SM twice, and a single CTA per SM loses a third of the rate:
+// 256 bins over 480 frames of 1280x720 took 295 us with 4 stages (one CTA per
+// SM), 191 us with kStagesWide (two CTAs), 203 us with 2 stages (two CTAs).
+constexpr int kStagesWide = 3;
+constexpr int kCellStages = COFIE_CELL_STAGES;
 constexpr int kGroupBytes = 48;            // 16 RGB pixels
 constexpr int kChunkGroups = COFIE_K1_CHUNK_GROUPS;
 constexpr int kChunkBytes = kChunkGroups * kGroupBytes;  // 24 KiB by default
@@ -208,12 +213,11 @@ struct ChunkCursor {
   }
 };
 
-template <int kBin>
+template <int kBin, int kS>
 __global__ void __launch_bounds__(Shape<kBin>::threads) hist_fast_kernel(SegTable segs, HistArgs a, LumaConsts L,
                                                                          uint32_t* __restrict__ hist,
                                                                          uint32_t* __restrict__ err) {
   constexpr int kCW = Shape<kBin>::warps, kNC = Shape<kBin>::consumers, kNT = Shape<kBin>::threads;
-  constexpr int kS = Shape<kBin>::stages;
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ SegLite sseg[kMaxSegs];
   uint8_t* ring = smem;
@@ -428,65 +432,63 @@ __global__ void __launch_bounds__(kGenericThreads) hist_generic_kernel(SegTable 
 
 }  // namespace
 
-size_t hist_smem_bytes(uint32_t bins) {
-  return static_cast<size_t>(kStages) * kChunkBytes + static_cast<size_t>(bins) * 32 * 4 + 2 * kStages * 8;
+static size_t hist_smem_bytes(uint32_t bins, int stages) {
+  return static_cast<size_t>(stages) * kChunkBytes + static_cast<size_t>(bins) * 32 * 4 + 2 * stages * 8;
 }
 
 static size_t cells_smem_bytes() {
-  constexpr int kS = Shape<kCells>::stages;
-  return static_cast<size_t>(kS) * kChunkBytes + static_cast<size_t>(kMaxBins) * 4 + 2 * kS * 8;
+  return static_cast<size_t>(kCellStages) * kChunkBytes + static_cast<size_t>(kMaxBins) * 4 + 2 * kCellStages * 8;
 }
 
-static int configure(int bin_path, uint32_t bins) {
-  const size_t smem = hist_smem_bytes(bins);
-  cudaError_t e = (bin_path == kBinFast)
-                      ? cudaFuncSetAttribute(hist_fast_kernel<kBinFast>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             static_cast<int>(smem))
-                      : cudaFuncSetAttribute(hist_fast_kernel<kBinTwoStep>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-  return e == cudaSuccess ? 0 : -1;
+static auto hist_fast_variant(int bin_path, int stages) {
+  return bin_path == kBinFast
+             ? (stages == kStages ? hist_fast_kernel<kBinFast, kStages> : hist_fast_kernel<kBinFast, kStagesWide>)
+             : (stages == kStages ? hist_fast_kernel<kBinTwoStep, kStages> : hist_fast_kernel<kBinTwoStep, kStagesWide>);
 }
 
-int hist_blocks_per_sm(int bin_path, uint32_t bins) {
-  if (configure(bin_path, bins) != 0) return -1;
+// CTAs of the variant resident on an SM, or -1 on error.
+static int hist_occupancy(int bin_path, uint32_t bins, int stages) {
+  const auto kernel = hist_fast_variant(bin_path, stages);
+  const int limit = static_cast<int>(hist_smem_bytes(kMaxBins, stages));  // for every handle's bins: the limit is the kernel's
   int n = 0;
-  const size_t smem = hist_smem_bytes(bins);
-  cudaError_t e = (bin_path == kBinFast)
-                      ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, hist_fast_kernel<kBinFast>, kThreads, smem)
-                      : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, hist_fast_kernel<kBinTwoStep>, kThreads, smem);
-  return e == cudaSuccess ? n : -1;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, limit) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, kThreads, hist_smem_bytes(bins, stages)) != cudaSuccess)
+    return -1;
+  return n;
+}
+
+int hist_blocks_per_sm(int bin_path, uint32_t bins, int* stages) {
+  *stages = kStages;
+  const int n = hist_occupancy(bin_path, bins, kStages);
+  if (n != 1) return n;
+  const int wide = hist_occupancy(bin_path, bins, kStagesWide);
+  if (wide < 2) return n;
+  *stages = kStagesWide;
+  return wide;
 }
 
 uint32_t hist_chunk_groups() { return kChunkGroups; }
 
 int cells_blocks_per_sm() {
+  const auto kernel = hist_fast_kernel<kCells, kCellStages>;
   const size_t smem = cells_smem_bytes();
-  if (cudaFuncSetAttribute(hist_fast_kernel<kCells>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(smem)) != cudaSuccess)
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
     return -1;
   int n = 0;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, hist_fast_kernel<kCells>, Shape<kCells>::threads, smem) ==
-                 cudaSuccess
-             ? n
-             : -1;
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, Shape<kCells>::threads, smem) == cudaSuccess ? n : -1;
 }
 
 cudaError_t launch_cells_fast(const SegTable& segs, const HistArgs& a, const LumaConsts& lc, uint32_t* cells,
                               uint32_t* err, int grid, cudaStream_t st, bool pdl) {
-  const cudaError_t e = launch_dependent(pdl, hist_fast_kernel<kCells>, dim3(grid), dim3(Shape<kCells>::threads),
-                                         cells_smem_bytes(), st, segs, a, lc, cells, err);
+  const cudaError_t e = launch_dependent(pdl, hist_fast_kernel<kCells, kCellStages>, dim3(grid),
+                                         dim3(Shape<kCells>::threads), cells_smem_bytes(), st, segs, a, lc, cells, err);
   return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
-cudaError_t launch_hist_fast(const SegTable& segs, const HistArgs& a, const LumaConsts& lc, int bin_path,
+cudaError_t launch_hist_fast(const SegTable& segs, const HistArgs& a, const LumaConsts& lc, int bin_path, int stages,
                              uint32_t* hist, uint32_t* err, int grid, cudaStream_t st, bool pdl) {
-  const size_t smem = hist_smem_bytes(lc.bins);
-  const cudaError_t e =
-      bin_path == kBinFast
-          ? launch_dependent(pdl, hist_fast_kernel<kBinFast>, dim3(grid), dim3(kThreads), smem, st, segs, a, lc, hist,
-                             err)
-          : launch_dependent(pdl, hist_fast_kernel<kBinTwoStep>, dim3(grid), dim3(kThreads), smem, st, segs, a, lc,
-                             hist, err);
+  const cudaError_t e = launch_dependent(pdl, hist_fast_variant(bin_path, stages), dim3(grid), dim3(kThreads),
+                                         hist_smem_bytes(lc.bins, stages), st, segs, a, lc, hist, err);
   return e == cudaSuccess ? cudaGetLastError() : e;
 }
 

@@ -90,3 +90,17 @@ def test_batched_calls_across_the_boundaries(n_sms):
         assert np.array_equal(kg, ko), (s, np.flatnonzero(kg != ko)[:10])
         assert np.all(np.abs(outs[s][0].cpu().numpy().astype(np.float64) - so) <= 1e-6 * so)
     f.close()
+
+
+def test_bin_counts_around_the_ring_sizes():
+    """The bulk-copy kernel runs a shorter ring once the counters of many bins
+    would leave one CTA per SM: bin counts on both sides of that, on handles
+    alive together."""
+    from paper_2609_03675_gb300 import NGFF
+    w, h, T = 1280, 720, 60  # past the generic kernel's window
+    spec = synth.medium(seed=78).with_(width=w, height=h, frames=T, mean_scene_len=15)
+    fr = synth.generate(spec)
+    dev = torch.from_numpy(fr).cuda()
+    handles = {b: NGFF(w, h, bins=b, tau=0.05) for b in (256, 128, 127, 112, 64, 200)}
+    for b, f in handles.items():
+        assert_parity(run_stream(f, dev, [T]), oracle_run(fr, O.Params(w, h, bins=b, tau=0.05)), 0.05, f"B={b}")
