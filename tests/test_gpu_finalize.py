@@ -83,6 +83,32 @@ def test_gather_rejects_bad_index_without_reading_it():
     f.status()  # the error word was cleared; the handle keeps working
 
 
+@pytest.mark.parametrize("pinned", [False, True])
+@pytest.mark.parametrize("w,h", [(1, 1), (2, 3), (5, 1), (16, 1), (7, 3), (16, 2), (33, 11), (341, 17), (683, 24)])
+def test_gather_any_size_and_alignment(w, h, pinned):
+    """Frame sizes below, at and past the 16-byte words and a block's share of
+    them, frames and output at every offset mod 16, the buffer's first and
+    last frames among those taken; bytes around the output stay untouched."""
+    n, fb = 6, 3 * w * h
+    rng = np.random.default_rng(fb)
+    fr = rng.integers(0, 256, n * fb, dtype=np.uint8)
+    sel = [5, 0, 3, 3, 1]
+    idx = torch.tensor(sel, dtype=torch.int32, device="cuda")
+    want = fr.reshape(n, fb)[sel].reshape(-1)
+    f = _ngff(w, h)
+    for a in range(16):
+        for b in (0, a, (5 * a + 3) % 16, 15):
+            src = torch.empty(a + n * fb, dtype=torch.uint8)
+            src[a:] = torch.from_numpy(fr)
+            src = src.pin_memory() if pinned else src.cuda()
+            dst = torch.full((b + len(sel) * fb + 16,), 7, dtype=torch.uint8, device="cuda")
+            f.gather(src[a:], idx, out=dst[b:b + len(sel) * fb])
+            got = dst.cpu().numpy()
+            assert np.array_equal(got[b:b + len(want)], want), (a, b)
+            assert (got[:b] == 7).all() and (got[b + len(want):] == 7).all(), (a, b)
+    f.status()
+
+
 @pytest.mark.parametrize("w,h", [(160, 96), (17, 13)])
 def test_gather_from_pinned_host_frames(w, h):
     """Frames pushed from pinned host memory and gathered from it (the kernel
