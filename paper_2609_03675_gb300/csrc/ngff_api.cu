@@ -90,6 +90,8 @@ struct cofie_ngff {
   uint32_t* d_idx = nullptr;    // candidate indices when the caller's idx_out is host memory (allocated on first use)
   uint64_t dirty_rows = 0;      // histogram rows [0, dirty_rows) may be nonzero
   uint16_t* d_map = nullptr;    // a shard's gap map
+  uint8_t* d_chain_maps = nullptr;   // the tiled selection's maps
+  uint32_t* d_chain_flags = nullptr; // its two counters, then a flag per tile
   struct {                      // the shard prepared and not yet committed
     bool ready = false;
     uint32_t stream = 0, n_halo = 0, n = 0;
@@ -433,11 +435,13 @@ int run_segments(cofie_ngff* h, const SegTable& segs, cudaStream_t st, bool keep
   SelectArgs sa = select_args(h);
   uint32_t longest = 0;
   for (uint32_t i = 0; i < segs.count; ++i) longest = segs.s[i].n > longest ? segs.s[i].n : longest;
-  // small pushes clear their rows inside the selection kernel (saving a
-  // launch); large ones with one device-wide memset after the selection
+  // pushes clear their rows inside the selection kernel (saving a launch),
+  // except where the window and scan kernels or the L_max = 0 walk decide
+  // them: there one memset after the selection does
   const bool walk = h->p.l_max > 0 && h->p.l_max <= select_walk_max_lmax() && longest <= select_walk_max_frames();
+  const bool chain = h->p.l_max > 0 && !walk && !sa.scd;
   const bool fused = longest <= select_small_max();
-  sa.zero_hist = ((walk || fused) && !keep_hist && h->p.l_max > 0) ? 1u : 0u;
+  sa.zero_hist = ((walk || chain || fused) && !keep_hist && h->p.l_max > 0) ? 1u : 0u;
   cudaEvent_t es0 = nullptr, es1 = nullptr;
   if (timed && take_pair(h->ev_sel, h->ev_sel_used, &es0, &es1)) cudaEventRecord(es0, st);
   if (h->p.l_max == 0) {  // no forced retention: the rule walked in frame order
@@ -446,6 +450,11 @@ int run_segments(cofie_ngff* h, const SegTable& segs, cudaStream_t st, bool keep
     h->n_select += 1;
   } else if (walk) {  // distances and the rule walked in frame order, in one small launch per stream
     e = launch_select_walk(segs, sa, h->d_hist, h->d_ring, h->d_state, st, !ev0);
+    if (e != cudaSuccess) return h->cuda_fail(e, "selection kernel launch");
+    h->n_select += 1;
+  } else if (chain) {  // tiles of frames, each linked to those before it by their gap maps
+    const ChainArgs ca{h->d_chain_maps, h->d_chain_flags + 2, h->d_chain_flags, h->d_err, kTimeoutNs, 0u, 0u};
+    e = launch_select_chain(segs, sa, ca, h->num_sms, h->d_hist, h->d_ring, h->d_state, st, !ev0);
     if (e != cudaSuccess) return h->cuda_fail(e, "selection kernel launch");
     h->n_select += 1;
   } else if (fused) {  // distances and scan in one launch
@@ -592,7 +601,8 @@ void free_handle(cofie_ngff* h) {
   DeviceGuard guard(h->device);
   cudaDeviceSynchronize();
   void* bufs[] = {h->d_hist,     h->d_l1,       h->d_mask,  h->d_ring, h->d_state, h->d_scores, h->d_keep,
-                  h->d_err,      h->d_stage[0], h->d_stage[1], h->d_count, h->d_map, h->d_cells, h->d_record, h->d_idx};
+                  h->d_err,      h->d_stage[0], h->d_stage[1], h->d_count, h->d_map, h->d_cells, h->d_record, h->d_idx,
+                  h->d_chain_maps, h->d_chain_flags};
   for (void* b : bufs)
     if (b) cudaFree(b);
   for (cudaEvent_t ev : h->ev_pool) cudaEventDestroy(ev);
@@ -752,6 +762,10 @@ int cofie_ngff_create(const cofie_ngff_params* p, cofie_ngff_t** out) {
   if (e == cudaSuccess) e = dalloc(&h->d_count, 1);
   if (e == cudaSuccess) e = dalloc(&h->d_map, COFIE_NGFF_MAX_LMAX);
   if (e == cudaSuccess) e = dalloc(&h->d_record, S * h->rec_words);
+  const bool chained = p->l_max > 0 && p->signal != COFIE_SIGNAL_SCD;
+  const size_t chain_flags = chain_max_tiles(p->max_frames_per_push) + size_t(2);
+  if (e == cudaSuccess && chained) e = dalloc(&h->d_chain_maps, chain_flags * 32 * h->mask_words);
+  if (e == cudaSuccess && chained) e = dalloc(&h->d_chain_flags, chain_flags);
   if (e == cudaSuccess && p->signal == COFIE_SIGNAL_DHASH) {
     e = dalloc(&h->d_cells, F * 72);
     if (e == cudaSuccess) e = cudaMemset(h->d_cells, 0, F * 72 * sizeof(uint32_t));
@@ -771,6 +785,8 @@ int cofie_ngff_create(const cofie_ngff_params* p, cofie_ngff_t** out) {
     e = cudaEventCreateWithFlags(&h->ev_copied[i], cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_free[i], cudaEventDisableTiming);
   }
+  if (e == cudaSuccess && chained) e = cudaMemset(h->d_chain_flags, 0, chain_flags * sizeof(uint32_t));
+  if (e == cudaSuccess && chained) e = chain_prepare();
   if (e == cudaSuccess && p->l_max > 0) e = scan_prepare(h->mask_words, p->l_max);
   if (e == cudaSuccess && h->bin_path >= 0) {
     const int per_sm = hist_blocks_per_sm(h->bin_path, p->bins, &h->hist_stages);
@@ -1157,18 +1173,19 @@ int cofie_ngff_status(cofie_ngff_t* h, void* cuda_stream) {
   if (e != cudaSuccess) return h->cuda_fail(e, "error word read");
   if (checked_build()) {  // the index checks of every kernel file (checked builds only)
     const uint32_t b = take_bounds_errors_hist() | take_bounds_errors_features() | take_bounds_errors_select() |
-                       take_bounds_errors_lazy() | take_bounds_errors_finalize();
+                       take_bounds_errors_chain() | take_bounds_errors_lazy() | take_bounds_errors_finalize();
     if (b) word |= kErrBounds;
   }
   if (word) {
     cudaMemset(h->d_err, 0, sizeof word);
-    char buf[128];
+    char buf[256];
     snprintf(buf, sizeof buf,
-             "device-side failure (error bits 0x%x: 1/2/4 a wait ran out, 8 a bad gather index, 16 an index check "
+             "device-side failure (error bits 0x%x: 1/2/4/64 a wait ran out, 8 a bad gather index, 16 an index check "
              "of the checked build, 32 candidates of a stream past its retention record)",
              word);
-    return h->fail((word & (kErrConsumerTimeout | kErrProducerTimeout | kErrDrainTimeout)) ? COFIE_ETIMEOUT
-                                                                                          : COFIE_EDEVICE,
+    return h->fail((word & (kErrConsumerTimeout | kErrProducerTimeout | kErrDrainTimeout | kErrChainTimeout))
+                       ? COFIE_ETIMEOUT
+                       : COFIE_EDEVICE,
                    buf);
   }
   return COFIE_OK;

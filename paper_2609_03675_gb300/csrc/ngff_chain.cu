@@ -1,0 +1,367 @@
+// Selection of larger pushes in one launch (CoFiE Sec. 3.2, Eqs. 2-5): novelty
+// distances, the rule and the outputs of a push of any number of frames.
+//
+// The gap g = t - r(t) lies in [1, L_max] (Eq. 5's second term retains a frame
+// whenever g reaches L_max), so a frame's keep decision is one bit per
+// possible gap, and a run of frames is a map from the gap before it to the gap
+// after it. The push is cut into tiles of `tile` frames of one stream. A CTA
+// takes one tile:
+//   1. the tile's histogram rows and the L_max rows before them (this push's
+//      rows, or the stream's ring) are copied into shared memory (kStaged) and
+//      the windowed distances L1[j][k-1] = sum_b |c_t - c_{t-k}| and keep bits
+//      computed there, a warp per frame, lane = lag;
+//   2. the tile's gap map is composed for every entry gap at once (thread =
+//      entry gap), noting the gap before each frame, and published;
+//   3. the entry gap follows from the stream's gap and the maps of the tiles
+//      before this one, of which at most kLookBack are composed: a tile
+//      further on takes the known exit gap of the tile kLookBack before it;
+//   4. scores, keep codes and record bits are written. The stream's last tile
+//      also stores the ring and the state. Rows that no later tile reads are
+//      zeroed for the next push.
+// Tiles are handed out by a ticket in stream order, so a CTA only ever waits
+// for tiles that are already running: no co-residency is needed. Every wait is
+// bounded; one that runs out sets an error bit and goes on with an arbitrary
+// gap. The last CTA to finish returns tickets and flags to zero.
+//
+// Bound by latency: a push's tables are a few MB at most, in L2. This kernel
+// took the place of three dependent launches, one for the distances, one
+// single-CTA scan of the tables that it wrote and a memset of the rows: 4096
+// frames of 224x224 (B = 32, L_max = 30) pushed in 116 instead of 135 us, 480
+// of 1280x720 (B = 256, L_max = 60) in 211 instead of 236 us.
+#include <algorithm>
+
+#include "ngff_common.cuh"
+
+namespace cofie {
+namespace {
+
+constexpr int kChainThreads = 256;
+constexpr uint32_t kChainWarps = kChainThreads / 32;
+constexpr uint32_t kLookBack = 128;            // tiles whose maps a tile composes
+constexpr size_t kChainSmemMax = 200 * 1024;   // rows are staged when everything fits
+constexpr uint32_t kChainMaxTile = 32;
+
+static_assert(kMaxLmax <= kChainThreads, "a thread per entry gap");
+static_assert(kLookBack <= kChainThreads, "a thread per flag");
+
+// A tile's flag: 0 nothing yet, 1 its map is published, (g << 2) | 3 also its
+// exit gap g is known.
+constexpr uint32_t kMapReady = 1u, kExitKnown = 3u;
+
+__device__ __forceinline__ uint64_t now_ns() {
+  uint64_t t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+
+__device__ __forceinline__ uint32_t flag_acquire(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+
+__device__ __forceinline__ void flag_release(uint32_t* p, uint32_t v) {
+  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
+// The flag once it has all bits of `want`, or 0 after timeout_ns.
+__device__ __forceinline__ uint32_t flag_wait(const uint32_t* p, uint32_t want, uint64_t timeout_ns) {
+  uint32_t v = flag_acquire(p);
+  if ((v & want) == want) return v;
+  const uint64_t t0 = now_ns();
+  for (;;) {
+#pragma unroll 1
+    for (int i = 0; i < 64; ++i) {
+      v = flag_acquire(p);
+      if ((v & want) == want) return v;
+    }
+    if (now_ns() - t0 > timeout_ns) return 0;
+  }
+}
+
+__device__ __forceinline__ uint32_t absdiff(uint32_t a, uint32_t b) { return a > b ? a - b : b - a; }
+
+// sum_b |x_b - y_b| by one thread; 16-byte words from the rotated word `rot`
+// on (lanes that read rows B words apart then touch distinct banks).
+template <bool kVec4>
+__device__ __forceinline__ uint32_t row_l1(const uint32_t* x, const uint32_t* y, uint32_t B, uint32_t rot, uint32_t kind) {
+  uint32_t d = 0;
+  if (kVec4) {
+    const uint4* x4 = reinterpret_cast<const uint4*>(x);
+    const uint4* y4 = reinterpret_cast<const uint4*>(y);
+    uint32_t q = rot;
+#pragma unroll 8
+    for (uint32_t i = 0; i < B / 4; ++i) {
+      const uint4 u = x4[q], v = y4[q];
+      d += absdiff(u.x, v.x) + absdiff(u.y, v.y) + absdiff(u.z, v.z) + absdiff(u.w, v.w);
+      if (++q == B / 4) q = 0;
+    }
+  } else if (kind == 1) {  // Hamming distance of bit vectors (dHash)
+    for (uint32_t b = 0; b < B; ++b) d += __popc(x[b] ^ y[b]);
+  } else {
+#pragma unroll 4
+    for (uint32_t b = 0; b < B; ++b) d += absdiff(x[b], y[b]);
+  }
+  return d;
+}
+
+// Shared memory, in words: [rows][l1][masks][maps of kLookBack tiles][gap
+// before each frame, by entry gap][the warps' composed maps]
+struct ChainLayout {
+  uint32_t rows, l1, mask, maps, gaps, comp, words;
+  __host__ __device__ ChainLayout(uint32_t tile, uint32_t l_max, uint32_t mask_words, uint32_t bins, bool staged) {
+    const uint32_t map_words = 8 * mask_words;  // 32 mask_words entries of one byte
+    rows = 0;
+    l1 = rows + (staged ? (l_max + tile) * bins : 0);
+    mask = l1 + tile * l_max;
+    maps = mask + tile * mask_words;
+    gaps = maps + kLookBack * map_words;
+    comp = gaps + tile * map_words;
+    words = comp + kChainWarps * map_words;
+  }
+};
+
+template <bool kVec4, bool kStaged>
+__global__ void __launch_bounds__(kChainThreads) select_chain_kernel(SegTable segs, SelectArgs a, ChainArgs c,
+                                                                     uint32_t* __restrict__ hist,
+                                                                     uint32_t* __restrict__ ring,
+                                                                     StreamState* __restrict__ state) {
+  extern __shared__ __align__(16) uint32_t csm[];
+  __shared__ uint32_t s_seg, s_k, s_base, s_entry, s_bad;
+  __shared__ uint32_t s_flag0;
+  const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const uint32_t B = a.bins, L = a.l_max, W = a.mask_words, F = c.tile;
+  const uint32_t stride = 32 * W;  // bytes of a map
+  const ChainLayout lay(F, L, W, B, kStaged);
+  uint32_t* rows = csm + lay.rows;
+  uint32_t* l1 = csm + lay.l1;
+  uint32_t* mask = csm + lay.mask;
+  uint8_t* maps = reinterpret_cast<uint8_t*>(csm + lay.maps);
+  uint8_t* gaps = reinterpret_cast<uint8_t*>(csm + lay.gaps);
+  uint8_t* comp = reinterpret_cast<uint8_t*>(csm + lay.comp);
+
+  pdl_trigger();  // the next push's first-stage kernel may be scheduled; it waits for this grid before its work
+  pdl_wait();     // every device read follows: the histograms, and the state and counters the last push left
+  if (tid == 0) {
+    const uint32_t t = atomicAdd(&c.sync[0], 1u);
+    uint32_t seg = 0, base = 0, n = (segs.s[0].n + F - 1) / F;
+    while (t >= base + n && seg + 1 < segs.count) {
+      base += n;
+      n = (segs.s[++seg].n + F - 1) / F;
+    }
+    s_seg = seg;
+    s_base = base;
+    s_k = t - base;
+    s_bad = 0;
+  }
+  __syncthreads();
+  const Segment& sg = segs.s[s_seg];
+  const uint32_t k_tile = s_k, base = s_base, n = sg.n, j0 = k_tile * F, n_tiles = (n + F - 1) / F;
+  if (!COFIE_BOUND(j0 < n && base + k_tile < c.n_tiles)) return;
+  const uint32_t fn = min(F, n - j0);
+  const bool last_tile = k_tile + 1 == n_tiles;
+  const unsigned long long t0 = state[sg.stream].t;
+  const uint32_t t0_slot = static_cast<uint32_t>(t0 % L);  // ring slot of the push's first frame
+  uint32_t* hist_s = hist + static_cast<uint64_t>(sg.row0) * B;
+  uint32_t* ring_s = ring + static_cast<uint64_t>(sg.stream) * L * B;
+  // row i of the staged rows is the push's frame j0 - L + i; frames before the
+  // push lie in the ring (slots of frames that never were are read, not used)
+  const auto row_of = [&](int32_t jj) -> const uint32_t* {
+    if (jj >= 0) return hist_s + static_cast<uint64_t>(jj) * B;
+    uint32_t slot = t0_slot + static_cast<uint32_t>(jj + static_cast<int32_t>(L));  // jj >= -L
+    if (slot >= L) slot -= L;
+    return ring_s + static_cast<uint64_t>(slot) * B;
+  };
+
+  // 1. rows, distances, keep bits
+  if (kStaged) {
+    if (kVec4) {
+      const uint32_t nq = B / 4;
+#pragma unroll 4
+      for (uint32_t i = tid; i < (L + fn) * nq; i += kChainThreads) {
+        const uint32_t r = i / nq;
+        reinterpret_cast<uint4*>(rows)[i] =
+            reinterpret_cast<const uint4*>(row_of(static_cast<int32_t>(j0 + r) - static_cast<int32_t>(L)))[i - r * nq];
+      }
+    } else {
+      for (uint32_t i = tid; i < (L + fn) * B; i += kChainThreads) {
+        const uint32_t r = i / B;
+        rows[i] = row_of(static_cast<int32_t>(j0 + r) - static_cast<int32_t>(L))[i - r * B];
+      }
+    }
+    __syncthreads();
+  }
+  const uint32_t rot = kStaged && kVec4 ? lane % max(B / 4, 1u) : 0u;
+  for (uint32_t j = warp; j < fn; j += kChainWarps) {
+    const unsigned long long t = t0 + j0 + j;
+    const uint32_t* ct = kStaged ? rows + (L + j) * B : row_of(static_cast<int32_t>(j0 + j));
+    uint32_t l_adj = 0;
+    for (uint32_t w = 0; w < W; ++w) {
+      const uint32_t k = 32 * w + lane + 1;
+      const bool valid = k <= L && k <= t;
+      const uint32_t* src = ct;
+      if (valid) src = kStaged ? ct - k * B : row_of(static_cast<int32_t>(j0 + j) - static_cast<int32_t>(k));
+      uint32_t d = row_l1<kVec4>(ct, src, B, rot, a.dist_kind);
+      if (!valid) d = 0;
+      if (w == 0) l_adj = __shfl_sync(0xffffffffu, d, 0);  // lag 1
+      if (k <= L) l1[j * L + k - 1] = d;
+      // fp32(max) / 2N >= tau exactly when max >= x_tau (the smallest such numerator)
+      const bool keep = k <= L && (max(l_adj, d) >= a.x_tau || k >= L);
+      const uint32_t m = __ballot_sync(0xffffffffu, keep);
+      if (lane == 0) mask[j * W + w] = m;
+    }
+  }
+  __syncthreads();
+
+  // 2. the tile's gap map (entry and exit gaps less one, in bytes)
+  uint8_t* my_map = c.maps + static_cast<uint64_t>(base + k_tile) * stride;
+  uint32_t exit_gap = 0;
+  if (tid < L) {
+    uint32_t g = tid;
+    for (uint32_t j = 0; j < fn; ++j) {
+      gaps[j * stride + tid] = static_cast<uint8_t>(g);
+      const bool keep = (mask[j * W + (g >> 5)] >> (g & 31)) & 1u;
+      g = (keep || t0 + j0 + j == 0) ? 0u : g + 1u;  // the stream's first frame restarts the gap
+    }
+    (void)COFIE_BOUND(g < L);
+    exit_gap = g;
+    if (!last_tile) __stcg(my_map + tid, static_cast<uint8_t>(g));
+  }
+  __syncthreads();
+  if (tid == 0 && !last_tile) {
+    __threadfence();
+    flag_release(c.flags + base + k_tile, kMapReady);
+  }
+
+  // 3. the entry gap
+  const uint32_t lo = k_tile > kLookBack ? k_tile - kLookBack : 0;  // the earliest tile looked at
+  const uint32_t first = lo > 0 ? lo + 1 : 0;                       // the earliest whose map is composed
+  const uint32_t m = k_tile - first;
+  if (k_tile > 0) {
+    if (tid < k_tile - lo) {
+      const uint32_t v = flag_wait(c.flags + base + lo + tid, lo > 0 && tid == 0 ? kExitKnown : kMapReady, c.timeout_ns);
+      if (v == 0) s_bad = 1;
+      if (tid == 0) s_flag0 = v;
+    }
+    __syncthreads();
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(c.maps + static_cast<uint64_t>(base + first) * stride);
+    for (uint32_t i = tid; i < m * (stride / 4); i += kChainThreads) reinterpret_cast<uint32_t*>(maps)[i] = __ldcg(src + i);
+    __syncthreads();
+    // a warp composes a run of maps for every entry gap, one thread chains the runs
+    const uint32_t per = (m + kChainWarps - 1) / kChainWarps, a0 = min(warp * per, m), a1 = min(a0 + per, m);
+    for (uint32_t e = lane; e < L; e += 32) {
+      uint32_t g = e;
+      for (uint32_t i = a0; i < a1; ++i) g = maps[i * stride + g];
+      comp[warp * stride + e] = static_cast<uint8_t>(g);
+    }
+    __syncthreads();
+  }
+  if (tid == 0) {
+    uint32_t g = lo > 0 ? s_flag0 >> 2 : state[sg.stream].g;
+    if (t0 == 0 && lo == 0) g = 1;
+    if (g < 1 || g > L) g = L;  // the state only ever holds [1, L]
+    --g;
+    if (k_tile > 0)
+      for (uint32_t w = 0; w < kChainWarps; ++w) g = comp[w * stride + g];
+    if (s_bad) {
+      atomicOr(c.err, kErrChainTimeout);
+      g = L - 1;
+    }
+    s_entry = g;
+  }
+  __syncthreads();
+  const uint32_t entry = s_entry;
+  if (tid == entry) {  // this thread's exit gap is the tile's
+    if (last_tile) {
+      state[sg.stream].t = t0 + n;
+      state[sg.stream].g = exit_gap + 1;
+      if (t0 == 0) state[sg.stream].acc = 0;
+    } else {
+      flag_release(c.flags + base + k_tile, ((exit_gap + 1) << 2) | kExitKnown);
+    }
+  }
+
+  // 4. outputs, the record, ring and state, and the rows cleared
+  if (warp == 0) {
+    const uint32_t j = lane;
+    bool kept = false;
+    if (j < fn) {
+      float s = 0.0f;
+      uint8_t code = 3;
+      if (t0 + j0 + j != 0) {
+        uint32_t g = gaps[j * stride + entry];
+        if (!COFIE_BOUND(g < L)) g = 0;
+        s = __fdiv_rn(static_cast<float>(max(l1[j * L], l1[j * L + g])), a.two_n);
+        code = s >= a.tau ? 1 : (g + 1 >= L ? 2 : 0);
+      }
+      if (sg.scores) sg.scores[j0 + j] = s;
+      if (sg.keep) sg.keep[j0 + j] = code;
+      kept = code != 0;
+    }
+    const uint32_t bits = __ballot_sync(0xffffffffu, kept);
+    if (lane == 0 && a.record)
+      record_bits(a.record + static_cast<uint64_t>(sg.stream) * a.rec_words, a.rec_words, t0 + j0, bits);
+  }
+  if (last_tile) {  // every tile before this one has read the ring and the state: their flags were seen
+    const uint32_t keep_n = min(n, L);
+    for (uint32_t i = tid; i < keep_n * B; i += kChainThreads) {
+      const uint32_t r = i / B, b = i - r * B, jj = n - keep_n + r;
+      const uint32_t v = kStaged ? rows[(L + jj - j0) * B + b] : hist_s[static_cast<uint64_t>(jj) * B + b];
+      ring_s[static_cast<uint64_t>((t0_slot + jj) % L) * B + b] = v;
+    }
+    __syncthreads();  // the rows below have been copied
+  }
+  if (a.zero_hist) {
+    // tiles up to this one have read their rows, later ones read from L rows
+    // before them on
+    const uint32_t z0 = j0 > L ? j0 - L : 0, z1 = last_tile ? n : (j0 + F > L ? j0 + F - L : 0);
+    for (uint64_t i = static_cast<uint64_t>(z0) * B + tid; i < static_cast<uint64_t>(z1) * B; i += kChainThreads) hist_s[i] = 0;
+  }
+  __syncthreads();
+  if (tid == 0) s_bad = atomicAdd(&c.sync[1], 1u) == c.n_tiles - 1;
+  __syncthreads();
+  if (s_bad) {  // the last CTA: nobody waits any more
+    for (uint32_t i = tid; i < c.n_tiles; i += kChainThreads) c.flags[i] = 0;
+    if (tid < 2) c.sync[tid] = 0;
+  }
+}
+
+// Frames per tile: as few as keep the grid at about one CTA per SM, so that a
+// short push spreads over the SMs and a long one composes few maps.
+uint32_t chain_tile(const SegTable& segs, int num_sms) {
+  uint32_t tile = 8;
+  while (tile < kChainMaxTile && segs.rows > tile * static_cast<uint32_t>(num_sms)) tile *= 2;
+  return tile;
+}
+
+}  // namespace
+
+uint32_t chain_max_tiles(uint32_t max_frames) { return max_frames / 8 + kMaxSegs + 1; }
+
+cudaError_t chain_prepare() {
+  for (const auto k : {select_chain_kernel<true, true>, select_chain_kernel<false, true>, select_chain_kernel<true, false>,
+                       select_chain_kernel<false, false>}) {
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kChainSmemMax);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+cudaError_t launch_select_chain(const SegTable& segs, const SelectArgs& a, ChainArgs c, int num_sms, uint32_t* hist,
+                                uint32_t* ring, StreamState* state, cudaStream_t st, bool pdl) {
+  c.tile = chain_tile(segs, num_sms);
+  c.n_tiles = 0;
+  for (uint32_t i = 0; i < segs.count; ++i) c.n_tiles += (segs.s[i].n + c.tile - 1) / c.tile;
+  const bool staged = ChainLayout(c.tile, a.l_max, a.mask_words, a.bins, true).words * sizeof(uint32_t) <= kChainSmemMax;
+  const size_t smem = ChainLayout(c.tile, a.l_max, a.mask_words, a.bins, staged).words * sizeof(uint32_t);
+  const bool vec = a.bins % 4 == 0 && a.dist_kind == 0;
+  const auto kernel = vec ? (staged ? select_chain_kernel<true, true> : select_chain_kernel<true, false>)
+                          : (staged ? select_chain_kernel<false, true> : select_chain_kernel<false, false>);
+  const cudaError_t e = launch_dependent(pdl, kernel, dim3(c.n_tiles), dim3(kChainThreads), smem, st, segs, a, c, hist,
+                                         ring, state);
+  return e == cudaSuccess ? cudaGetLastError() : e;
+}
+
+uint32_t take_bounds_errors_chain() { return take_local_bounds_errors(); }
+
+}  // namespace cofie

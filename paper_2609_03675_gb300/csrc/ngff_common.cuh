@@ -132,6 +132,7 @@ uint32_t take_bounds_errors_hist();
 uint32_t take_bounds_errors_features();
 uint32_t take_bounds_errors_select();
 uint32_t take_bounds_errors_lazy();
+uint32_t take_bounds_errors_chain();
 uint32_t take_bounds_errors_finalize();
 bool checked_build();
 
@@ -142,6 +143,7 @@ constexpr uint32_t kErrDrainTimeout = 4u;
 constexpr uint32_t kErrBadIndex = 8u;  // a gather index outside the frame buffer
 constexpr uint32_t kErrBounds = 16u;   // checked build: an index check failed
 constexpr uint32_t kErrRecord = 32u;   // candidates of a stream that has run past its retention record
+constexpr uint32_t kErrChainTimeout = 64u;  // a selection tile's wait for the tiles before it
 
 struct HistArgs {
   uint64_t frame_bytes;      // 3 W H
@@ -174,6 +176,18 @@ struct SelectArgs {
   // the streams' retention records ([streams][rec_words]; nullptr: none)
   uint32_t* record;
   uint32_t rec_words;
+};
+
+// The tiled selection's workspace: gap maps and flags of a push's tiles, and
+// the ticket and the count of finished tiles (flags and counters are zero
+// between pushes).
+struct ChainArgs {
+  uint8_t* maps;
+  uint32_t* flags;
+  uint32_t* sync;
+  uint32_t* err;
+  uint64_t timeout_ns;
+  uint32_t tile, n_tiles;  // frames per tile, tiles of the launch (set by it)
 };
 
 // Sets the record bits of retained frames: bit i of `bits` stands for frame
@@ -248,6 +262,11 @@ cudaError_t launch_select_walk(const SegTable& segs, const SelectArgs& a, uint32
                                StreamState* state, cudaStream_t st, bool pdl = false);
 cudaError_t launch_cells_any(const SegTable& segs, const FeatArgs& fa, const LumaConsts& lc, uint32_t* cells,
                              int num_sms, cudaStream_t st, bool pdl = false);
+// pushes with L_max > 0 and no scene changes that are too large for the walk
+uint32_t chain_max_tiles(uint32_t max_frames);
+cudaError_t chain_prepare();
+cudaError_t launch_select_chain(const SegTable& segs, const SelectArgs& a, ChainArgs c, int num_sms, uint32_t* hist,
+                                uint32_t* ring, StreamState* state, cudaStream_t st, bool pdl = false);
 int cells_blocks_per_sm();
 cudaError_t launch_cells_fast(const SegTable& segs, const HistArgs& a, const LumaConsts& lc, uint32_t* cells,
                               uint32_t* err, int grid, cudaStream_t st, bool pdl = false);

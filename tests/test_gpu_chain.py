@@ -1,0 +1,74 @@
+"""The selection of larger pushes: tiles of frames linked by their gap maps.
+Pushes around the tile sizes and around the number of tiles that a tile looks
+back on, rows staged in shared memory and not, one and several mask words,
+ring and state carried from push to push, and batches of unequal lengths,
+against the oracle's single pass."""
+import numpy as np
+import pytest
+import torch
+
+import oracle as O
+import synth
+from tests.gpu_helpers import assert_parity, oracle_run, run_stream
+
+pytestmark = pytest.mark.gpu
+
+W, H = 32, 8
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+
+
+def _frames(T, seed=41, mean=9):
+    return synth.generate(synth.medium(seed=seed).with_(width=W, height=H, frames=T, mean_scene_len=mean))
+
+
+# 8 frames per tile up to 1216 on 152 SMs, 16 up to 2432, 32 beyond; a tile looks back on 128
+PUSHES = [[65], [66, 72, 1], [1033, 1024], [1216, 1217], [2432, 70], [2433, 5000], [3, 9001]]
+
+
+@pytest.mark.parametrize("bins,l_max,tau", [(32, 30, 0.15), (32, 1, 0.30), (7, 33, 0.20), (256, 60, 0.50), (32, 256, 0.35),
+                                            (256, 256, 0.60), (4, 64, 2.0), (32, 30, 0.0)])
+@pytest.mark.parametrize("sizes", PUSHES)
+def test_pushes_match_the_oracle(sizes, bins, l_max, tau):
+    from paper_2609_03675_gb300 import NGFF
+    fr = _frames(sum(sizes))
+    want = oracle_run(fr, O.Params(W, H, bins=bins, l_max=l_max, tau=tau))
+    dev = torch.from_numpy(fr).cuda()
+    f = NGFF(W, H, bins=bins, l_max=l_max, tau=tau, max_frames_per_push=max(sizes))
+    assert_parity(run_stream(f, dev, sizes), want, tau, "with histograms")
+    f.reset()
+    got = [f.push(part) for part in torch.split(dev, sizes)]  # rows cleared by the selection itself
+    torch.cuda.synchronize()
+    f.status()
+    assert np.array_equal(torch.cat([k for _, k in got]).cpu().numpy(), want[2])
+    assert torch.equal(f.candidates().cpu(), torch.from_numpy(O.load().candidates(want[2], 4).astype(np.int32)))
+
+
+@pytest.mark.parametrize("bins,l_max", [(32, 30), (256, 256)])
+def test_batches_of_unequal_lengths(bins, l_max):
+    from paper_2609_03675_gb300 import NGFF
+    calls = [(0, 1, 65, 700), (9, 70, 0, 8), (130, 64, 3, 1500)]
+    fr = [_frames(sum(c[s] for c in calls) or 1, seed=50 + s) for s in range(4)]
+    tau = 0.2
+    f = NGFF(W, H, bins=bins, l_max=l_max, tau=tau, max_streams=4)
+    dev = [torch.from_numpy(x).cuda() for x in fr]
+    outs = [(torch.empty(len(x), dtype=torch.float32, device="cuda"), torch.empty(len(x), dtype=torch.uint8, device="cuda"))
+            for x in fr]
+    at = [0] * 4
+    for c in calls:
+        items = []
+        for s in range(4):
+            a, b = at[s], at[s] + c[s]
+            items.append((s, dev[s][a:b], outs[s][0][a:b], outs[s][1][a:b]))
+            at[s] = b
+        f.push_batch(items)
+    torch.cuda.synchronize()
+    f.status()
+    for s in range(4):
+        _, so, ko = oracle_run(fr[s], O.Params(W, H, bins=bins, l_max=l_max, tau=tau))
+        assert np.array_equal(outs[s][1].cpu().numpy(), ko), s
+        assert np.all(np.abs(outs[s][0].cpu().numpy().astype(np.float64) - so) <= 1e-6 * so), s
