@@ -92,9 +92,7 @@ typedef struct cofie_ngff cofie_ngff_t;
  *   l_max             L_max in sampled-frame indices, 0..256; default 30 (App. B.2).
  *                     0 turns the forced retention (Eq. 5's second term) off:
  *                     frames are then kept only as first, novelty or scene
- *                     change, the rule is walked in frame order (by windows
- *                     of 32 frames between keeps, one warp per stream), and
- *                     the stream cannot be sharded.
+ *                     change, and the stream cannot be sharded.
  *   m_min             M_min, used by cofie_ngff_candidates only; default 4 (App. B.2).
  *   tau               tau_h, any non-NaN float; default 0.30f (App. B.2).
  *   luma_w, luma_den  grayscale weights (wR, wG, wB) / den; each weight <= 65535,

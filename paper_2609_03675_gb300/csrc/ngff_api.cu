@@ -90,6 +90,7 @@ struct cofie_ngff {
   uint32_t* d_idx = nullptr;    // candidate indices when the caller's idx_out is host memory (allocated on first use)
   uint64_t dirty_rows = 0;      // histogram rows [0, dirty_rows) may be nonzero
   uint16_t* d_map = nullptr;    // a shard's gap map
+  uint32_t* d_lazy = nullptr;        // L_max = 0: scratch of larger pushes
   uint8_t* d_chain_maps = nullptr;   // the tiled selection's maps
   uint32_t* d_chain_flags = nullptr; // its two counters, then a flag per tile
   struct {                      // the shard prepared and not yet committed
@@ -436,18 +437,24 @@ int run_segments(cofie_ngff* h, const SegTable& segs, cudaStream_t st, bool keep
   uint32_t longest = 0;
   for (uint32_t i = 0; i < segs.count; ++i) longest = segs.s[i].n > longest ? segs.s[i].n : longest;
   // pushes clear their rows inside the selection kernel (saving a launch),
-  // except where the window and scan kernels or the L_max = 0 walk decide
-  // them: there one memset after the selection does
+  // except where the window and scan kernels or the larger selection without
+  // forced retention decide them: there one memset after the selection does
   const bool walk = h->p.l_max > 0 && h->p.l_max <= select_walk_max_lmax() && longest <= select_walk_max_frames();
   const bool chain = h->p.l_max > 0 && !walk && !sa.scd;
   const bool fused = longest <= select_small_max();
-  sa.zero_hist = ((walk || chain || fused) && !keep_hist && h->p.l_max > 0) ? 1u : 0u;
+  const bool lazy_walk = h->p.l_max == 0 && lazy_walk_fits(longest, h->fw);
+  sa.zero_hist = ((walk || chain || lazy_walk || (fused && h->p.l_max > 0)) && !keep_hist) ? 1u : 0u;
   cudaEvent_t es0 = nullptr, es1 = nullptr;
   if (timed && take_pair(h->ev_sel, h->ev_sel_used, &es0, &es1)) cudaEventRecord(es0, st);
-  if (h->p.l_max == 0) {  // no forced retention: the rule walked in frame order
-    e = launch_lazy_select(segs, sa, h->d_hist, h->d_ring, h->d_state, st, !ev0);
+  if (lazy_walk) {  // no forced retention, few frames
+    e = launch_lazy_walk(segs, sa, h->d_hist, h->d_ring, h->d_state, st, !ev0);
     if (e != cudaSuccess) return h->cuda_fail(e, "lazy selection kernel launch");
     h->n_select += 1;
+  } else if (h->p.l_max == 0) {  // no forced retention: links between references, the chain of them, the outputs
+    e = launch_lazy_select(segs, sa, h->d_lazy, h->p.max_frames_per_push, h->num_sms, h->d_hist, h->d_ring, h->d_state, st,
+                           !ev0);
+    if (e != cudaSuccess) return h->cuda_fail(e, "lazy selection kernel launch");
+    h->n_select += 3;
   } else if (walk) {  // distances and the rule walked in frame order, in one small launch per stream
     e = launch_select_walk(segs, sa, h->d_hist, h->d_ring, h->d_state, st, !ev0);
     if (e != cudaSuccess) return h->cuda_fail(e, "selection kernel launch");
@@ -602,7 +609,7 @@ void free_handle(cofie_ngff* h) {
   cudaDeviceSynchronize();
   void* bufs[] = {h->d_hist,     h->d_l1,       h->d_mask,  h->d_ring, h->d_state, h->d_scores, h->d_keep,
                   h->d_err,      h->d_stage[0], h->d_stage[1], h->d_count, h->d_map, h->d_cells, h->d_record, h->d_idx,
-                  h->d_chain_maps, h->d_chain_flags};
+                  h->d_chain_maps, h->d_chain_flags, h->d_lazy};
   for (void* b : bufs)
     if (b) cudaFree(b);
   for (cudaEvent_t ev : h->ev_pool) cudaEventDestroy(ev);
@@ -764,6 +771,7 @@ int cofie_ngff_create(const cofie_ngff_params* p, cofie_ngff_t** out) {
   if (e == cudaSuccess) e = dalloc(&h->d_record, S * h->rec_words);
   const bool chained = p->l_max > 0 && p->signal != COFIE_SIGNAL_SCD;
   const size_t chain_flags = chain_max_tiles(p->max_frames_per_push) + size_t(2);
+  if (e == cudaSuccess && p->l_max == 0) e = dalloc(&h->d_lazy, lazy_scratch_words(p->max_frames_per_push, h->fw));
   if (e == cudaSuccess && chained) e = dalloc(&h->d_chain_maps, chain_flags * 32 * h->mask_words);
   if (e == cudaSuccess && chained) e = dalloc(&h->d_chain_flags, chain_flags);
   if (e == cudaSuccess && p->signal == COFIE_SIGNAL_DHASH) {
@@ -787,6 +795,7 @@ int cofie_ngff_create(const cofie_ngff_params* p, cofie_ngff_t** out) {
   }
   if (e == cudaSuccess && chained) e = cudaMemset(h->d_chain_flags, 0, chain_flags * sizeof(uint32_t));
   if (e == cudaSuccess && chained) e = chain_prepare();
+  if (e == cudaSuccess && p->l_max == 0) e = lazy_prepare();
   if (e == cudaSuccess && p->l_max > 0) e = scan_prepare(h->mask_words, p->l_max);
   if (e == cudaSuccess && h->bin_path >= 0) {
     const int per_sm = hist_blocks_per_sm(h->bin_path, p->bins, &h->hist_stages);

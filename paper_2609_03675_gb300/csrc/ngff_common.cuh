@@ -190,6 +190,17 @@ struct ChainArgs {
   uint32_t tile, n_tiles;  // frames per tile, tiles of the launch (set by it)
 };
 
+// Scratch of the selection of larger pushes without forced retention: per row
+// of the push the adjacent distance, the frame that would follow it as a
+// reference, and its own reference; per segment the first successor of the
+// stream's reference, whether the stream began with the push, and a copy of
+// the reference's row.
+struct LazyArgs {
+  uint32_t *adj, *next, *ref;
+  uint32_t *next_pre, *first, *old_ref;
+  uint32_t tile, stage_rows;  // references per CTA of the next kernel, rows that it stages
+};
+
 // Sets the record bits of retained frames: bit i of `bits` stands for frame
 // t_first + i of the stream whose record is `rec` (rec_words words). Frames
 // at or past the record's end are not recorded. One thread per call.
@@ -273,8 +284,14 @@ cudaError_t launch_cells_fast(const SegTable& segs, const HistArgs& a, const Lum
 cudaError_t launch_dhash_finish(uint32_t* cells, uint32_t rows, const FeatArgs& fa, uint32_t* bits, cudaStream_t st,
                                 bool pdl = false);
 cudaError_t launch_wait_probe(uint64_t timeout_ns, uint32_t* err, cudaStream_t st);
-cudaError_t launch_lazy_select(const SegTable& segs, const SelectArgs& a, const uint32_t* feat, uint32_t* ring,
-                               StreamState* state, cudaStream_t st, bool pdl = false);
+// L_max = 0: pushes whose longest piece of a stream one CTA decides, and larger ones
+bool lazy_walk_fits(uint32_t longest, uint32_t bins);
+size_t lazy_scratch_words(uint32_t max_frames, uint32_t bins);
+cudaError_t lazy_prepare();
+cudaError_t launch_lazy_walk(const SegTable& segs, const SelectArgs& a, uint32_t* feat, uint32_t* ring, StreamState* state,
+                             cudaStream_t st, bool pdl = false);
+cudaError_t launch_lazy_select(const SegTable& segs, const SelectArgs& a, uint32_t* scratch, uint32_t max_frames, int num_sms,
+                               const uint32_t* feat, uint32_t* ring, StreamState* state, cudaStream_t st, bool pdl = false);
 cudaError_t launch_debug_bins(const uint8_t* px, uint64_t n_groups, const LumaConsts& lc, int bin_path,
                               uint8_t* bins_out, cudaStream_t st);
 cudaError_t scan_prepare(uint32_t mask_words, uint32_t l_max);

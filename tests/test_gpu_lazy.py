@@ -114,3 +114,64 @@ def test_batch_of_streams_without_gap():
     for s in range(S):
         _, so, ko = O.load().run(frs[s], O.Params(w, h, tau=0.06, l_max=0))
         assert np.array_equal(torch.cat([k for _, k in outs[s]]).cpu().numpy(), ko), f"stream {s}"
+
+
+# Pushes on both sides of the single-kernel limit (192 frames, fewer with wide
+# rows) and of its ways to share out the pairs (16 frames), of the links'
+# tiles and staged rows (fewer with wide rows), and of the chain's passes of
+# 4096 frames; a still stream, whose links run past the staged rows, between
+# scenes; every frame kept.
+@pytest.mark.parametrize("bins,tau,still", [(32, 0.06, 0), (32, 0.06, 700), (256, 0.2, 300), (6, 0.1, 150), (32, 0.0, 0),
+                                            (64, 0.9, 0)])
+@pytest.mark.parametrize("scd", [False, True])
+@pytest.mark.parametrize("chunks", [[1, 16, 17, 7, 33, 2], [192, 193, 129, 64], [4096, 5], [3, 4097, 400],
+                                    [257, 1300, 66]])
+def test_links_and_chain(chunks, bins, tau, still, scd):
+    from paper_2609_03675_gb300 import NGFF, _abi
+    w, h, T = 32, 8, sum(chunks)
+    fr = _frames(w, h, T, seed=760 + bins + T, mean=7)
+    for a in range(100, T, 2 * still) if still else ():
+        fr[a:a + still] = fr[a]
+    p = O.Params(w, h, bins=bins, tau=tau, l_max=0)
+    kw = dict(bins=bins, tau=tau, l_max=0, max_frames_per_push=max(chunks))
+    if scd:
+        hist = np.stack([O.load().histogram(x, p) for x in fr])
+        sd = np.array([SC.l1(hist[t], hist[t - 1]) for t in range(1, T)]) / (2 * w * h)
+        sd = sd[sd > 0]
+        t_grad, t_cut = float(np.quantile(sd, 0.6)), float(np.quantile(sd, 0.97))
+        so, ko = SC.select(hist, p, t_cut, t_grad)
+        kw.update(signal=_abi.SIGNAL_SCD, scd_cut=t_cut, scd_gradual=t_grad)
+    else:
+        _, so, ko = O.load().run(fr, p)
+    f = NGFF(w, h, **kw)
+    got = [f.push(part) for part in torch.split(torch.from_numpy(fr).cuda(), chunks)]
+    torch.cuda.synchronize()
+    f.status()
+    kg = torch.cat([k for _, k in got]).cpu().numpy()
+    assert np.array_equal(kg, ko), np.flatnonzero(kg != ko)[:10]
+    assert (np.abs(torch.cat([s for s, _ in got]).cpu().numpy().astype(np.float64) - so) <= SCORE_RTOL * so).all()
+    assert torch.equal(f.candidates().cpu(), torch.from_numpy(O.load().candidates(ko, 4).astype(np.int32)))
+
+
+def test_batch_of_unequal_lengths_without_gap():
+    from paper_2609_03675_gb300 import NGFF
+    calls = [(0, 1, 65, 700), (9, 70, 0, 8), (1, 64, 3, 2)]
+    frs = [_frames(32, 8, sum(c[s] for c in calls), seed=790 + s, mean=6) for s in range(4)]
+    f = NGFF(32, 8, tau=0.06, l_max=0, max_streams=4)
+    dev = [torch.from_numpy(x).cuda() for x in frs]
+    outs = [(torch.empty(len(x), dtype=torch.float32, device="cuda"), torch.empty(len(x), dtype=torch.uint8, device="cuda"))
+            for x in frs]
+    at = [0] * 4
+    for c in calls:
+        items = []
+        for s in range(4):
+            a, b = at[s], at[s] + c[s]
+            items.append((s, dev[s][a:b], outs[s][0][a:b], outs[s][1][a:b]))
+            at[s] = b
+        f.push_batch(items)
+    torch.cuda.synchronize()
+    f.status()
+    for s in range(4):
+        _, so, ko = O.load().run(frs[s], O.Params(32, 8, tau=0.06, l_max=0))
+        assert np.array_equal(outs[s][1].cpu().numpy(), ko), s
+        assert (np.abs(outs[s][0].cpu().numpy().astype(np.float64) - so) <= SCORE_RTOL * so).all(), s
