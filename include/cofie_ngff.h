@@ -502,11 +502,11 @@ typedef struct {
 
 /* Scoring kernels: the paired-SM one (clusters of two CTAs, one M = 256 MMA
  * per pair) needs the text block (n_text, or for n_text > 256 its blocks,
- * which are padded to 32) rounded up to 16 to be a multiple of 32; AUTO takes
- * it when it applies and the 256-token tiles of a run either fit one per
- * co-resident pair (76 on GB300) or exceed one wave of the one-SM kernel (one
- * per SM). The results of the two agree up to the order of fp32 accumulation
- * inside the tensor cores. */
+ * which are padded to 32) rounded up to 16 to be a multiple of 32 when asked
+ * for as PAIR; AUTO pads the block for it and takes, run by run, the kernel
+ * that measured faster for the run's count of 256-token tiles, the text block
+ * and H_kv d_h. The results of the two agree up to the order of fp32
+ * accumulation inside the tensor cores. */
 #define COFIE_QER_KERNEL_AUTO 0
 #define COFIE_QER_KERNEL_ONE_SM 1
 #define COFIE_QER_KERNEL_PAIR 2

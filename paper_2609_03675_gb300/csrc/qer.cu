@@ -897,6 +897,29 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
   return fn;
 }
 
+// Which kernel scores a run of the automatic choice, from calls at 16 to 1024
+// tiles, D = 128, 512, 1024 and 32 to 256 text rows (us a call from a graph,
+// one-SM / paired):
+//   every tile can have a pair of its own, each SM half of its MMAs and keys:
+//     paired (D = 1024: 16 tiles of 32 rows 15.4 / 13.2, 64 tiles 16.4 / 15.5);
+//   up to one wave of the one-SM kernel: one-SM (100 tiles 17.6 / 21.1);
+//   beyond that, more than 128 rows and D past 256: paired, which reads q~ half
+//     as often per SM (1024 tiles of 256 rows: D = 1024 103.8 / 96.4, D = 512
+//     64.7 / 58.7);
+//   few rows or short dot products are bound by the keys' bytes, where a tile
+//     on one SM costs less set-up than on two (1024 tiles of 32 rows: D = 128
+//     23.2 / 32.1, D = 512 53.8 / 56.6, D = 1024 90.3 / 92.5), unless the one-SM
+//     kernel's last wave is at most half full and the waves before it are few
+//     against the length of a tile (D = 1024, 200 tiles 29.6 / 27.7, 512 tiles
+//     52.5 / 50.9; but D = 512, 512 tiles 34.2 / 35.9).
+bool pair_is_faster(uint32_t tiles, uint32_t D, uint32_t rows, uint32_t one_sm_grid, uint32_t pairs) {
+  if (tiles <= pairs) return true;
+  if (tiles <= one_sm_grid) return false;
+  if (rows > 128 && D > 256) return true;
+  const uint32_t waves = tiles / one_sm_grid, last = tiles % one_sm_grid;
+  return last > 0 && 2 * last <= one_sm_grid && waves * 256 <= D;
+}
+
 // 2-D bf16 tensor [rows][cols] (cols contiguous), boxes of 64 columns x box_rows.
 bool make_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows) {
   auto enc = tensor_map_encoder();
@@ -922,7 +945,8 @@ struct cofie_qer {
   // the text is scored in n_blk passes of per_blk tokens (the last may have
   // fewer), each padded to n_pad q~ rows; q~ holds n_blk * n_pad rows
   uint32_t n_blk = 1, per_blk = 0;
-  uint32_t n_pad = 0, D = 0, acc_cols = 0, n_buf = 1, n_stages = 0;
+  uint32_t n_pad = 0, n_pad_one = 0;  // n_pad_one: the rows that the one-SM kernel scores
+  uint32_t D = 0, acc_cols = 0, n_buf = 1, n_stages = 0;
   int grid = 0;          // persistent CTAs
   size_t smem = 0;       // dynamic shared memory per CTA
   bool pair = false;     // the paired-SM kernel (clusters of two CTAs)
@@ -1009,10 +1033,11 @@ int cofie_qer_create(const cofie_qer_params* p, cofie_qer_t** out) {
   h->D = static_cast<uint32_t>(D);
   h->n_blk = (p->n_text + kQerMaxN - 1) / kQerMaxN;  // balanced blocks of at most 256 tokens
   h->per_blk = (p->n_text + h->n_blk - 1) / h->n_blk;
-  // rows of a block: a multiple of 16 (the MMA's N step), of 32 when there are
-  // several blocks so that the paired kernel (half of q~ per CTA) stays open
-  const uint32_t row_step = h->n_blk > 1 ? 32u : 16u;
-  h->n_pad = (h->per_blk + row_step - 1) / row_step * row_step;
+  // rows of a block: a multiple of 16 (the MMA's N step) for the one-SM kernel,
+  // of 32 for the paired kernel, whose CTAs take half of q~ each; a call on the
+  // one-SM kernel leaves out the last 16 rows when they hold no text
+  h->n_pad = (h->per_blk + 31) / 32 * 32;
+  h->n_pad_one = h->n_blk > 1 ? h->n_pad : (h->per_blk + 15) / 16 * 16;
   h->acc_cols = 32;
   while (h->acc_cols < h->n_pad) h->acc_cols <<= 1;
   // Each tile needs two accumulators of acc_cols TMEM columns; double
@@ -1046,7 +1071,10 @@ int cofie_qer_create(const cofie_qer_params* p, cofie_qer_t** out) {
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, dev);
   if (e == cudaSuccess && (per_sm_ctas < 1 || per_sm_ctas > max_ctas_by_tmem)) e = cudaErrorInvalidConfiguration;
   h->grid = n_sms * (per_sm_ctas > 0 ? per_sm_ctas : 1);
-  if (e == cudaSuccess && p->kernel != COFIE_QER_KERNEL_ONE_SM && h->n_pad % 32 == 0) {
+  // asked for by name, the paired kernel takes a text block that rounds up to
+  // 32 rows by itself; the automatic choice has it for every query
+  if (e == cudaSuccess && (p->kernel == COFIE_QER_KERNEL_AUTO ||
+                           (p->kernel == COFIE_QER_KERNEL_PAIR && h->n_pad_one % 32 == 0))) {
     // the paired-SM kernel: one accumulator of acc_cols columns per buffer,
     // two buffers; the same TMEM residency rule through shared memory
     // two 64-wide K chunks per ring stage when D allows: every stage costs a
@@ -1139,13 +1167,11 @@ int cofie_qer_run(cofie_qer_t* h, const uint16_t* q, const uint16_t* k, uint32_t
   const uint64_t nv = static_cast<uint64_t>(n_frames) * p.tokens_per_frame;
   CUtensorMap map_k, map_q;
   const uint32_t tiles = static_cast<uint32_t>((nv + kQerTile - 1) / kQerTile);
-  // the paired kernel when asked for, or (automatic) when every tile gets a
-  // pair of its own (each tile's MMAs split over two SMs: 14 us against 18 us
-  // for up to 76 tiles) or the tiles exceed one wave of the one-SM kernel; in
-  // between (one wave of that kernel, two of the pairs) the two run alike
-  const bool pair_run = h->pair && (p.kernel == COFIE_QER_KERNEL_PAIR || tiles > static_cast<uint32_t>(h->grid) ||
-                                    tiles <= static_cast<uint32_t>(h->pair_clusters));
-  const uint32_t q_box = pair_run ? h->n_pad / 2 : h->n_pad;  // the pair's CTAs each stage half of q~
+  const bool pair_run =
+      h->pair && (p.kernel == COFIE_QER_KERNEL_PAIR ||
+                  pair_is_faster(tiles, h->D, h->n_pad, static_cast<uint32_t>(h->grid), static_cast<uint32_t>(h->pair_clusters)));
+  const uint32_t n_pad = pair_run ? h->n_pad : h->n_pad_one;
+  const uint32_t q_box = pair_run ? n_pad / 2 : n_pad;  // the pair's CTAs each stage half of q~
   if (!make_map(&map_k, k, nv, h->D, kQerM)) return h->fail(COFIE_ECUDA, "tensor map encoding failed");
   const uint32_t n_rows = h->n_blk * h->n_pad;
   if (p.head_dim % 8 == 0 && reinterpret_cast<uintptr_t>(q) % 16 == 0) {
@@ -1196,7 +1222,7 @@ int cofie_qer_run(cofie_qer_t* h, const uint16_t* q, const uint16_t* k, uint32_t
   // after the pass before them as usual (no programmatic launch), so each
   // reads that pass's maxima complete.
   for (uint32_t blk = 0; blk < h->n_blk; ++blk) {
-    if (!make_map(&map_q, h->d_qg + static_cast<size_t>(blk) * h->n_pad * h->D, h->n_pad, h->D, q_box))
+    if (!make_map(&map_q, h->d_qg + static_cast<size_t>(blk) * h->n_pad * h->D, n_pad, h->D, q_box))
       return h->fail(COFIE_ECUDA, "tensor map encoding failed");
     const uint32_t text_b = std::min(h->per_blk, p.n_text - blk * h->per_blk);  // real columns of this pass
     const uint32_t fold = blk > 0;
@@ -1209,7 +1235,7 @@ int cofie_qer_run(cofie_qer_t* h, const uint16_t* q, const uint16_t* k, uint32_t
       cfg.numAttrs = fold ? 1 : 2;
       const uint32_t n_chunks = h->D / kQerKChunk / h->pair_sub;
       cudaLaunchKernelEx(&cfg, h->pair_sub == 2 ? qer_score_pair<2> : qer_score_pair<1>, map_k, map_q,
-                         static_cast<uint32_t>(nv), text_b, h->n_pad, fold, h->acc_cols, h->pair_key_slots,
+                         static_cast<uint32_t>(nv), text_b, n_pad, fold, h->acc_cols, h->pair_key_slots,
                          kQerPairQSlots, n_chunks, tiles, h->d_colmax, h->d_err, 2000000000ull);
     } else {
       cfg.gridDim = dim3(grid, 1, 1);
@@ -1217,7 +1243,7 @@ int cofie_qer_run(cofie_qer_t* h, const uint16_t* q, const uint16_t* k, uint32_t
       cfg.dynamicSmemBytes = h->smem;
       cfg.attrs = attr;
       cfg.numAttrs = fold ? 0 : 1;
-      cudaLaunchKernelEx(&cfg, qer_score, map_k, map_q, static_cast<uint32_t>(nv), text_b, h->n_pad, fold,
+      cudaLaunchKernelEx(&cfg, qer_score, map_k, map_q, static_cast<uint32_t>(nv), text_b, n_pad, fold,
                          h->acc_cols, h->n_buf, h->n_stages, h->D / kQerKChunk, tiles, h->d_colmax, h->d_err,
                          2000000000ull);
     }
@@ -1225,7 +1251,7 @@ int cofie_qer_run(cofie_qer_t* h, const uint16_t* q, const uint16_t* k, uint32_t
   if (e1) cudaEventRecord(e1, st);
   if (!capturing) {
     h->launches += 1;
-    h->flops += 2.0 * n_rows * static_cast<double>(nv) * h->D;
+    h->flops += 2.0 * h->n_blk * n_pad * static_cast<double>(nv) * h->D;
     h->key_bytes += 2.0 * static_cast<double>(nv) * h->D * h->n_blk;  // each pass reads the keys
   }
   cfg.gridDim = dim3((n_frames + 7) / 8, 1, 1);

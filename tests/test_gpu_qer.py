@@ -228,3 +228,22 @@ def test_captured_call_replays_on_new_inputs(kernel):
         assert torch.equal(w, w_ref)
         assert int(kdev.item()) == sel_ref.numel()
         assert torch.equal(sel[: sel_ref.numel()], sel_ref)
+
+
+@pytest.mark.parametrize("n_text", [1, 8, 16, 40, 48, 70, 144, 200])
+@pytest.mark.parametrize("n_frames", [3, 120, 250])
+def test_any_text_length_on_the_automatic_choice(n_text, n_frames):
+    """Text blocks that do not round up to 32 rows by themselves: padded for
+    the paired kernel, not for the one-SM kernel, at frame counts where the
+    automatic choice takes the one or the other; asked for by name the paired
+    kernel still refuses them."""
+    from paper_2609_03675_gb300 import QER, NGFFError
+    spec = S.QerSpec(n_text=n_text, n_heads=8, n_kv_heads=2, head_dim=64, n_frames=n_frames, tokens_per_frame=256, seed=n_text)
+    check(spec, 0.3)
+    if (n_text + 15) // 16 * 16 % 32:
+        with pytest.raises(NGFFError):
+            QER(n_text, 8, 2, 64, 4, 8, 0.5, kernel=2)
+    exact = spec.with_(integer=True)
+    _, _, _, w1, s1 = _run_gpu(exact, 0.5, kernel=1)
+    _, _, _, w0, s0 = _run_gpu(exact, 0.5)
+    assert np.array_equal(w0, w1) and np.array_equal(s0, s1)
