@@ -32,8 +32,10 @@
 //                   a warp per frame;
 //   qer_rank        the k best frames by rank (ties to the lower index), a
 //                   warp per frame; the last CTA writes them in time order.
-// Every kernel after the first is a programmatic dependent of the one before
-// it, so its launch and set-up overlap that kernel's tail.
+// Every kernel is a programmatic dependent of the one before it (the first one
+// of the caller's, or of the call before), so its launch and set-up overlap
+// that kernel's tail; calls in a row take 2 us less each since the first
+// kernel is one too (128 frames of 40 text tokens 25.1 -> 23.4 us).
 // Every mbarrier wait is bounded by the global timer; a wait that runs out
 // sets an error bit, stops issuing, lets the work already issued finish
 // (bounded) and frees TMEM before the CTA exits.
@@ -301,7 +303,8 @@ __device__ __forceinline__ uint32_t qer_text_of_row(uint32_t p, uint32_t bp, uin
 __global__ void qer_prepare_q(const uint16_t* __restrict__ q, uint32_t n_text, uint32_t n_rows, uint32_t bp,
                               uint32_t per_blk, uint32_t H, uint32_t H_kv, uint32_t d,
                               __nv_bfloat16_raw* __restrict__ qg) {
-  grid_dependents_launch();  // the scoring kernel may start; its q~ loads wait for this grid
+  grid_dependency_wait();    // q, and the call before this one, which may still read q~ and the maxima
+  grid_dependents_launch();  // the scoring kernel may start: its keys are ready too; its q~ loads wait for this grid
   const uint32_t D = H_kv * d, G = H / H_kv;
   const uint64_t total = static_cast<uint64_t>(n_rows) * D;
   for (uint64_t e = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; e < total;
@@ -319,7 +322,8 @@ __global__ void qer_prepare_q(const uint16_t* __restrict__ q, uint32_t n_text, u
 // The same with 8 consecutive channels per thread (d % 8 == 0, 16-byte aligned q).
 __global__ void qer_prepare_q8(const uint4* __restrict__ q, uint32_t n_text, uint32_t n_rows, uint32_t bp,
                                uint32_t per_blk, uint32_t H, uint32_t H_kv, uint32_t d, uint4* __restrict__ qg) {
-  grid_dependents_launch();  // the scoring kernel may start; its q~ loads wait for this grid
+  grid_dependency_wait();    // q, and the call before this one, which may still read q~ and the maxima
+  grid_dependents_launch();  // the scoring kernel may start: its keys are ready too; its q~ loads wait for this grid
   const uint32_t d8 = d / 8, D8 = H_kv * d8, G = H / H_kv;
   const uint64_t total = static_cast<uint64_t>(n_rows) * D8;
   for (uint64_t e = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; e < total;
@@ -802,6 +806,7 @@ __global__ void __launch_bounds__(kRankThreads) qer_rank(const float* __restrict
   __shared__ uint32_t wsum[kWarps];
   __shared__ uint32_t s_total, s_last;
   __shared__ float sw[kRankTile];
+  grid_dependents_launch();  // the next call's first kernel may be scheduled; it waits for this grid before its work
   grid_dependency_wait();
   const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t f = blockIdx.x * kWarps + warp;
@@ -1177,11 +1182,11 @@ int cofie_qer_run(cofie_qer_t* h, const uint16_t* q, const uint16_t* k, uint32_t
   if (p.head_dim % 8 == 0 && reinterpret_cast<uintptr_t>(q) % 16 == 0) {
     const uint64_t n8 = static_cast<uint64_t>(n_rows) * h->D / 8;
     const uint32_t blocks = static_cast<uint32_t>(std::min<uint64_t>((n8 + 255) / 256, 1024));
-    qer_prepare_q8<<<blocks, 256, 0, st>>>(reinterpret_cast<const uint4*>(q), p.n_text, n_rows, h->n_pad, h->per_blk,
-                                           p.n_heads, p.n_kv_heads, p.head_dim, reinterpret_cast<uint4*>(h->d_qg));
+    launch_dependent(true, qer_prepare_q8, dim3(blocks), dim3(256), 0, st, reinterpret_cast<const uint4*>(q), p.n_text,
+                     n_rows, h->n_pad, h->per_blk, p.n_heads, p.n_kv_heads, p.head_dim, reinterpret_cast<uint4*>(h->d_qg));
   } else {
-    qer_prepare_q<<<256, 256, 0, st>>>(q, p.n_text, n_rows, h->n_pad, h->per_blk, p.n_heads, p.n_kv_heads,
-                                       p.head_dim, h->d_qg);
+    launch_dependent(true, qer_prepare_q, dim3(256), dim3(256), 0, st, q, p.n_text, n_rows, h->n_pad, h->per_blk, p.n_heads,
+                     p.n_kv_heads, p.head_dim, h->d_qg);
   }
   const uint32_t grid = tiles < static_cast<uint32_t>(h->grid) ? tiles : static_cast<uint32_t>(h->grid);
   const uint32_t kk = static_cast<uint32_t>(std::max(1.0, std::nearbyint(static_cast<double>(p.rho) * n_frames)));
@@ -1202,12 +1207,13 @@ int cofie_qer_run(cofie_qer_t* h, const uint16_t* q, const uint16_t* k, uint32_t
       cudaEventRecord(e0, st);
     }
   }
-  // The scoring, mean and ranking kernels are programmatic dependents of the
-  // kernel before them: each may be scheduled while its predecessor still
-  // runs, and waits for it (griddepcontrol.wait) only where it reads that
-  // kernel's output (the scoring kernel's q~ producer; every thread of the
-  // mean and ranking kernels). With the timing events in between, the
-  // scoring kernel's launch serialises as usual.
+  // Every kernel may be scheduled while its predecessor still runs, and waits
+  // for it (griddepcontrol.wait) where it reads what that kernel or one before
+  // it wrote: every thread of the first kernel, which lets the scoring kernel
+  // start only after its wait, so that the keys are ready when that one does;
+  // the scoring kernel's q~ producer; every thread of the mean and ranking
+  // kernels. With the timing events in between, the scoring kernel's launch
+  // serialises as usual.
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;

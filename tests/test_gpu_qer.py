@@ -247,3 +247,35 @@ def test_any_text_length_on_the_automatic_choice(n_text, n_frames):
     _, _, _, w1, s1 = _run_gpu(exact, 0.5, kernel=1)
     _, _, _, w0, s0 = _run_gpu(exact, 0.5)
     assert np.array_equal(w0, w1) and np.array_equal(s0, s1)
+
+
+@pytest.mark.parametrize("n_frames", [5, 90, 300])
+def test_inputs_written_by_the_kernel_before(n_frames):
+    """A call's first kernel may be scheduled while the kernel before it runs:
+    queries and keys that a caller's kernel writes just before the call, and
+    calls in a row that reuse the handle's scratch, must give what the same
+    inputs give at rest."""
+    from paper_2609_03675_gb300 import QER
+    specs = [S.QerSpec(n_text=40, n_heads=8, n_kv_heads=2, head_dim=64, n_frames=n_frames, tokens_per_frame=256, seed=s)
+             for s in range(3)]
+    data = [[torch.from_numpy(x.view(np.int16)).cuda().view(torch.bfloat16) for x in S.generate(sp)[:2]] for sp in specs]
+    g = QER(40, 8, 2, 64, n_frames, 256, 0.3)
+    want = []
+    for q, k in data:
+        w, sel = g.run(q, k)
+        want.append((w.clone(), sel.clone()))
+    q, k = torch.empty_like(data[0][0]), torch.empty_like(data[0][1])
+    n_sel = want[0][1].numel()
+    for _ in range(10):
+        got = []
+        for i in range(3):
+            w = torch.empty(n_frames, device="cuda")
+            sel, kd = torch.empty(n_frames, dtype=torch.int32, device="cuda"), torch.empty(1, dtype=torch.int32, device="cuda")
+            torch.mul(data[i][0], 1, out=q)
+            torch.mul(data[i][1], 1, out=k)
+            g.run_async(q, k, w, sel, kd)
+            got.append((w, sel))
+        torch.cuda.synchronize()
+        for (w, sel), (wo, so) in zip(got, want):
+            assert torch.equal(w, wo) and torch.equal(sel[:n_sel], so)
+    g.status()
