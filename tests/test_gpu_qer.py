@@ -279,3 +279,38 @@ def test_inputs_written_by_the_kernel_before(n_frames):
         for (w, sel), (wo, so) in zip(got, want):
             assert torch.equal(w, wo) and torch.equal(sel[:n_sel], so)
     g.status()
+
+
+@pytest.mark.parametrize("n", [1, 2, 31, 32, 33, 63, 64, 65, 300])
+@pytest.mark.parametrize("values", ["distinct", "ties", "equal", "special"])
+def test_selection_by_rank(n, values):
+    """The k best frames in time order on both sides of the count that one CTA
+    ranks, with distinct scores, ties across the cut, all equal, and with
+    infinities, both zeros and NaN: kept is every frame that fewer than k
+    others rank above, where a NaN compares as neither above nor below."""
+    from paper_2609_03675_gb300 import QER
+    rng = np.random.default_rng(n)
+    d, T = 64, 2
+    v = {"distinct": rng.permutation(n) - n / 2, "ties": rng.integers(-3, 4, n), "equal": np.full(n, 0.5),
+         "special": rng.choice([np.inf, -np.inf, 0.0, -0.0, 1.0, -1.0, 2.0], n)}[values].astype(np.float32)
+    v = (v.view(np.uint32) & 0xFFFF0000).view(np.float32)  # bf16 values
+    k = np.zeros((n, T, 1, d), dtype=np.float32)
+    k[:, :, 0, 0] = v[:, None]
+    if values == "special":  # +inf and -inf tokens in one frame: its mean is a NaN
+        k[rng.random(n) < 0.05, :, 0, 0] = (np.inf, -np.inf)
+    q = np.zeros((1, 1, d), dtype=np.float32)
+    q[0, 0, 0] = 1.0
+    for rho in (0.0, 0.1, 0.37, 1.0):
+        g = QER(1, 1, 1, d, n, T, rho)
+        w, sel = g.run(torch.from_numpy(q).to(torch.bfloat16).cuda(),
+                       torch.from_numpy(k.reshape(n * T, 1, d)).to(torch.bfloat16).cuda())
+        g.status()
+        w = w.cpu().numpy()
+        with np.errstate(invalid="ignore"):
+            want = (k[:, 0, 0, 0] + k[:, 1, 0, 0]) / np.float32(2) * np.float32(0.125)
+        assert np.array_equal(w, want, equal_nan=True)
+        kk = max(1, round(float(np.float32(rho)) * n))
+        real = np.flatnonzero(~np.isnan(w))
+        order = real[np.lexsort((real, -w[real]))][:kk]
+        assert np.array_equal(sel.cpu().numpy(), np.sort(np.concatenate([order, np.flatnonzero(np.isnan(w))])))
+        g.close()
