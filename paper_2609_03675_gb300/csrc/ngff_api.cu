@@ -36,7 +36,6 @@ thread_local std::string g_global_error;
 enum MemKind { kNull = 0, kDevice = 1, kHostPinned = 2, kHostPageable = 3 };
 
 constexpr uint64_t kDefaultStageBytes = 256ull << 20;
-constexpr uint32_t kSmallSliceGroups = 256;  // the generic kernel's slice for small launches (12 KiB of frame)
 constexpr uint32_t kDefaultRecordFrames = 1u << 20;  // frames per stream the retention record covers
 constexpr uint64_t kTimeoutNs = 2000000000ull;  // bounded device waits: 2 s
 constexpr size_t kMaxTimedEvents = 1u << 16;
@@ -69,8 +68,7 @@ struct cofie_ngff {
   int bin_path = -1;  // kBinFast, kBinTwoStep, or -1 (generic kernel only)
   bool size_fast = false;
   int hist_grid = 0;
-  int hist_stages = 0;   // K1's ring stages
-  uint64_t generic_wave = 0;  // CTAs of the generic kernel resident at once (0: never chosen over K1)
+  uint64_t generic_wave = 0;  // CTAs of the generic kernel resident at once
   int cells_grid = 0;    // the TMA kernel's grid for the spatial signals (0: not usable)
   unsigned long long x_tau = 0, x_cut = 0, x_grad = 0;  // integer forms of the fp32 decisions
   uint32_t m_gpr = 0, m_h = 0, m_gw = 0;  // its multiply-high divisors (16-pixel groups per row, height, grid columns)
@@ -335,34 +333,45 @@ cudaError_t launch_first_stage(cofie_ngff* h, const SegTable& segs, cudaStream_t
     if (e == cudaSuccess && dhash) e = launch_dhash_finish(h->d_cells, segs.rows, h->fa, h->d_hist, st, true);
     return e;
   }
-  // A launch whose generic grid fills the GPU in one wave of resident CTAs
-  // (at least two per SM, and at most an eighth of a second wave) runs the
-  // generic kernel: its CTAs start as SMs free and need no ring to fill,
-  // which K1's persistent CTAs, each with a fixed share of the chunks, pay on
-  // launches of that size (a batched call of 32 streams of 640x360: 23.2
-  // against 20.8 us). Launches too small for that window with the default
-  // slices take slices of kSmallSliceGroups groups if those land in it, as a
-  // programmatic dependent of the kernel before them (8-frame 448x448 pushes:
-  // 7.27 against 6.56 us per push); a grid near one wave stays an ordinary
-  // launch, because CTAs made resident ahead of time keep SMs the previous
-  // kernel still holds (the serving call went from 21 to 27 us). Smaller
-  // launches keep K1, whose CTAs are scheduled while the kernel before it
-  // runs; larger ones too, where the generic grid would end in a larger
-  // partial wave (a quarter of a wave already loses 6 %).
-  if (fast) {
-    const uint64_t lo = 2ull * h->num_sms, hi = h->generic_wave + h->generic_wave / 8;
-    const uint64_t gen_ctas = static_cast<uint64_t>(hist_generic_slices(h->npix)) * segs.rows;
-    if (gen_ctas >= lo && gen_ctas <= hi) return launch_hist_generic(segs, ha, h->lc, h->bin_path, h->d_hist, st);
-    const uint64_t small_ctas = static_cast<uint64_t>(hist_generic_slices(h->npix, kSmallSliceGroups)) * segs.rows;
-    if (gen_ctas < lo && small_ctas >= lo && small_ctas <= hi)
-      return launch_hist_generic(segs, ha, h->lc, h->bin_path, h->d_hist, st, kSmallSliceGroups, pdl);
+  // Which kernel, and the generic kernel's slices (16-pixel groups per CTA).
+  // Launches of up to kGenericBins bins, and of frames that K1 does not take:
+  //  - fewer than five CTAs of kWaveGroups per SM: slices of 256 groups, as a
+  //    programmatic dependent (pushes of 27 frames of 640x360 in 14.5 us on K1
+  //    12.4; one 4K frame 10.8 on K1, 8.7; 60 frames 19.6 with kWaveGroups,
+  //    18.3); with many bins to clear and fold 512 from 480,000 groups on (40
+  //    frames, 128 bins: 21.3 on kWaveGroups, 20.5 with 256, 19.6 with 512);
+  //  - up to one resident wave and an eighth of a second: kWaveGroups, as an
+  //    ordinary launch, whose CTAs start as SMs free (serving calls of 133
+  //    frames of 640x360: 24.3 us against 25.0 with half of that, 30.2 with
+  //    256 groups; made resident ahead of time they crowd the SMs that the
+  //    kernel before still holds);
+  //  - larger: slices short enough that the last wave's share is small, longer
+  //    with many bins (220 frames of 640x360: 105.7 on K1, 100.8 with 512, 104
+  //    with 1024; 600 1080p frames: 517 on K1, 544 with 512, 509 with 1024, 511
+  //    with 2048; 440 frames of 1280x720, 128 bins: 193 on K1, 188 with 2048).
+  // More bins on aligned frames: K1, whose persistent CTAs clear and fold their
+  // counters once per frame they touch (220 frames of 1280x720, 256 bins: 113
+  // us against 129 with 4096 groups), except launches that the generic grid
+  // covers in one wave, of kWaveGroups or of 256 groups.
+  constexpr uint32_t kWaveGroups = 2048, kGenericBins = 128;
+  const uint64_t sms = h->num_sms, hi = h->generic_wave + h->generic_wave / 8;
+  const uint64_t wave_ctas = static_cast<uint64_t>(hist_generic_slices(h->npix, kWaveGroups)) * segs.rows;
+  const auto generic = [&](uint32_t slice_groups, bool ahead) {
+    return launch_hist_generic(segs, ha, h->lc, h->bin_path, h->d_hist, st, slice_groups, ahead);
+  };
+  if (!fast || h->lc.bins <= kGenericBins) {
+    const uint64_t groups = static_cast<uint64_t>(h->npix / 16) * segs.rows;
+    const uint32_t longer = h->lc.bins > 128 ? 2 : (h->lc.bins > 64 ? 1 : 0);
+    if (wave_ctas < 5 * sms) return generic(longer && groups >= 480000 ? 512 : 256, pdl);
+    if (wave_ctas <= hi) return generic(kWaveGroups, false);
+    return generic((groups < 4000000 ? 512u : 1024u) << longer, false);
   }
-  if (fast) {
-    const uint64_t chunks = static_cast<uint64_t>(segs.rows) * ha.chunks_per_frame;
-    const int grid = static_cast<int>(chunks < static_cast<uint64_t>(h->hist_grid) ? chunks : h->hist_grid);
-    return launch_hist_fast(segs, ha, h->lc, h->bin_path, h->hist_stages, h->d_hist, h->d_err, grid, st, pdl);
-  }
-  return launch_hist_generic(segs, ha, h->lc, h->bin_path, h->d_hist, st);
+  const uint64_t small_ctas = static_cast<uint64_t>(hist_generic_slices(h->npix, 256)) * segs.rows;
+  if (wave_ctas >= 2 * sms && wave_ctas <= hi) return generic(kWaveGroups, false);
+  if (wave_ctas < 2 * sms && small_ctas >= 2 * sms && small_ctas <= hi) return generic(256, pdl);
+  const uint64_t chunks = static_cast<uint64_t>(segs.rows) * ha.chunks_per_frame;
+  const int grid = static_cast<int>(chunks < static_cast<uint64_t>(h->hist_grid) ? chunks : h->hist_grid);
+  return launch_hist_fast(segs, ha, h->lc, h->bin_path, h->d_hist, h->d_err, grid, st, pdl);
 }
 
 // The smallest numerator x with fp32(x) / den >= thr, or 2^64 - 1 if none.
@@ -798,9 +807,11 @@ int cofie_ngff_create(const cofie_ngff_params* p, cofie_ngff_t** out) {
   if (e == cudaSuccess && p->l_max == 0) e = lazy_prepare();
   if (e == cudaSuccess && p->l_max > 0) e = scan_prepare(h->mask_words, p->l_max);
   if (e == cudaSuccess && h->bin_path >= 0) {
-    const int per_sm = hist_blocks_per_sm(h->bin_path, p->bins, &h->hist_stages);
+    const int per_sm = hist_blocks_per_sm(h->bin_path, p->bins);
     if (per_sm <= 0) e = cudaGetLastError() != cudaSuccess ? cudaErrorInvalidConfiguration : cudaErrorInvalidValue;
     h->hist_grid = h->num_sms * (per_sm > 0 ? per_sm : 1);
+  }
+  if (e == cudaSuccess) {
     const int gen_per_sm = hist_generic_blocks_per_sm(h->bin_path, p->bins);
     if (gen_per_sm < 0) cudaGetLastError();
     h->generic_wave = gen_per_sm > 0 ? static_cast<uint64_t>(h->num_sms) * gen_per_sm : 0;

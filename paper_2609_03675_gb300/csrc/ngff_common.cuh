@@ -246,18 +246,16 @@ inline bool injected_alloc_failure() {
 }
 
 // Launchers (stream-ordered; return the launch error).
-// K1's resident CTAs per SM (-1 on error) and the ring stages that give them
-int hist_blocks_per_sm(int bin_path, uint32_t bins, int* stages);
+int hist_blocks_per_sm(int bin_path, uint32_t bins);  // K1's resident CTAs (-1 on error)
 uint32_t hist_chunk_groups();
-cudaError_t launch_hist_fast(const SegTable& segs, const HistArgs& a, const LumaConsts& lc, int bin_path, int stages,
+cudaError_t launch_hist_fast(const SegTable& segs, const HistArgs& a, const LumaConsts& lc, int bin_path,
                              uint32_t* hist, uint32_t* err, int grid, cudaStream_t st, bool pdl = false);
-// The generic kernel over CTAs of slice_groups 16-pixel groups (0: the
-// default 2048); with pdl a programmatic dependent of the kernel before it.
+// The generic kernel over CTAs of at most slice_groups 16-pixel groups (a
+// multiple of 256); with pdl a programmatic dependent of the kernel before it.
 cudaError_t launch_hist_generic(const SegTable& segs, const HistArgs& a, const LumaConsts& lc, int bin_path,
-                                uint32_t* hist, cudaStream_t st, uint32_t slice_groups = 0, bool pdl = false);
-// the generic kernel's CTAs per frame (slices of slice_groups groups, 0: the
-// default), and its resident CTAs per SM (-1 on error)
-uint32_t hist_generic_slices(uint32_t npix, uint32_t slice_groups = 0);
+                                uint32_t* hist, cudaStream_t st, uint32_t slice_groups, bool pdl = false);
+// the generic kernel's CTAs per frame, and its resident CTAs per SM (-1 on error)
+uint32_t hist_generic_slices(uint32_t npix, uint32_t slice_groups);
 int hist_generic_blocks_per_sm(int bin_path, uint32_t bins);
 cudaError_t launch_window(const SegTable& segs, const SelectArgs& a, const uint32_t* hist, const uint32_t* ring,
                           const StreamState* state, uint32_t* l1, uint32_t* mask, cudaStream_t st, bool pdl = false);

@@ -5,11 +5,15 @@
 // reading), bin = floor(Y B / 256), count[bin] += 1. Integer arithmetic only,
 // so the histogram is independent of summation order and bit-exact.
 //
+// Two kernels count them: the generic kernel below (any frame), which serves
+// histograms of up to 128 bins, and the fast kernel for more bins and for the
+// spatial signals, whose larger tables it clears and folds less often.
+//
 // Fast kernel (frames of a multiple of 16 pixels, 16-byte aligned):
 //   - a persistent grid; each CTA owns a contiguous range of 24 KiB chunks of
 //     the push (a chunk never crosses a frame boundary);
 //   - one producer thread streams chunks HBM -> shared memory with 1-D bulk
-//     async copies (cp.async.bulk, the TMA engine) into a 4-stage ring
+//     async copies (cp.async.bulk, the TMA engine) into a 3-stage ring
 //     guarded by mbarriers (full: transaction bytes, empty: consumer warps);
 //   - 4 consumer warps read 48-byte groups (16 RGB pixels) with three 128-bit
 //     shared loads at a 48-byte stride (conflict-free), form the luma sums
@@ -26,22 +30,26 @@
 // Every mbarrier wait is bounded (globaltimer); a wait that runs out sets a
 // bit in the error word, stops issuing work and returns without leaving bulk
 // copies in flight.
+#include <algorithm>
+
 #include "ngff_device.cuh"
 
 namespace cofie {
 namespace {
 
 // Tuning constants (compile-time overridable for sweeps). Measured on GB300
-// over the 1080p stream: 4 consumer warps (one per SM sub-partition) with two
-// CTAs per SM stream at ~7.59 TB/s; 3 or 5 warps (uneven over the
-// sub-partitions) lose 8-20 %, 8 warps lose 8 %, and any shape that leaves
-// one CTA per SM loses 25-40 %. The L2 evict-first hint makes no measurable
-// difference; the default policy is kept.
+// over the 1080p stream with 32 bins: 4 consumer warps (one per SM
+// sub-partition) with two CTAs per SM stream at ~7.59 TB/s; 3 or 5 warps
+// (uneven over the sub-partitions) lose 8-20 %, 8 warps lose 8 %, and any shape
+// that leaves one CTA per SM loses 25-40 %. So three ring stages: with 256 bins
+// (32 KiB of counters) four leave one CTA per SM, 480 frames of 1280x720 in 295
+// us against 191, two stages take 203. The L2 evict-first hint makes no
+// measurable difference; the default policy is kept.
 #ifndef COFIE_K1_CONSUMER_WARPS
 #define COFIE_K1_CONSUMER_WARPS 4
 #endif
 #ifndef COFIE_K1_STAGES
-#define COFIE_K1_STAGES 4
+#define COFIE_K1_STAGES 3
 #endif
 #ifndef COFIE_K1_CHUNK_GROUPS
 #define COFIE_K1_CHUNK_GROUPS 512
@@ -68,14 +76,8 @@ struct Shape {
   static constexpr int warps = kBin == kCells ? kCellWarps : kConsumerWarps;
   static constexpr int consumers = warps * 32;
   static constexpr int threads = consumers + 32;
+  static constexpr int stages = kBin == kCells ? COFIE_CELL_STAGES : COFIE_K1_STAGES;
 };
-constexpr int kStages = COFIE_K1_STAGES;
-// With many bins the counters (128 bytes a bin) and a ring of kStages no
-// longer fit an SM twice, and a single CTA per SM loses a third of the rate:
-// 256 bins over 480 frames of 1280x720 took 295 us with 4 stages (one CTA per
-// SM), 191 us with kStagesWide (two CTAs), 203 us with 2 stages (two CTAs).
-constexpr int kStagesWide = 3;
-constexpr int kCellStages = COFIE_CELL_STAGES;
 constexpr int kGroupBytes = 48;            // 16 RGB pixels
 constexpr int kChunkGroups = COFIE_K1_CHUNK_GROUPS;
 constexpr int kChunkBytes = kChunkGroups * kGroupBytes;  // 24 KiB by default
@@ -213,11 +215,12 @@ struct ChunkCursor {
   }
 };
 
-template <int kBin, int kS>
+template <int kBin>
 __global__ void __launch_bounds__(Shape<kBin>::threads) hist_fast_kernel(SegTable segs, HistArgs a, LumaConsts L,
                                                                          uint32_t* __restrict__ hist,
                                                                          uint32_t* __restrict__ err) {
   constexpr int kCW = Shape<kBin>::warps, kNC = Shape<kBin>::consumers, kNT = Shape<kBin>::threads;
+  constexpr int kS = Shape<kBin>::stages;
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ SegLite sseg[kMaxSegs];
   uint8_t* ring = smem;
@@ -349,9 +352,14 @@ __global__ void __launch_bounds__(Shape<kBin>::threads) hist_fast_kernel(SegTabl
   }
 }
 
-// Generic kernel: any frame size or alignment (frames whose pixel count is
-// not a multiple of 16, or that do not start on a 16-byte boundary). Grid
-// (slices, rows): CTA x of row r counts slice x of frame r. A frame's pixels
+// Generic kernel: any frame size or alignment. Grid (slices, rows, rows past a
+// dimension's limit): a CTA counts one slice of one frame. With eight CTAs per SM and nothing between a load and
+// its counts but registers it streams as fast as the fast kernel's ring or
+// faster, most of all over small frames, where the ring's chunks end ragged
+// (600 1080p frames 509 against 517 us, 4096 of 224x224 110 against 119, of
+// 96x112 46 against 54); 128 or 512 threads, four groups per turn of the loop
+// and 256-byte L2 requests were slower, one group a turn faster in small
+// launches and slower in serving calls (22.6 against 23.2 us). A frame's pixels
 // split into a prologue of p_a < 16 pixels, an interior of whole 16-pixel
 // groups that each start on a 16-byte boundary (p_a is the first pixel whose
 // address is 16-byte aligned: frame + 3 p_a = 0 mod 16), and an epilogue of
@@ -361,7 +369,7 @@ __global__ void __launch_bounds__(Shape<kBin>::threads) hist_fast_kernel(SegTabl
 // go to lane-private shared counters cnt[bin][lane] (bank = lane), folded
 // into the frame's row with one global atomic per bin per CTA.
 constexpr int kGenericThreads = 256;
-constexpr uint32_t kGenericGroupsPerCta = 2048;  // 32768 pixels per CTA, unless the launch asks for fewer
+constexpr uint32_t kGenericGridRows = 65535;
 constexpr int kGenericDiv = 3;                   // no verified multiply-high: Y = v / den
 
 template <int kBin>
@@ -381,7 +389,8 @@ __global__ void __launch_bounds__(kGenericThreads) hist_generic_kernel(SegTable 
                                                                       uint32_t* __restrict__ hist) {
   extern __shared__ __align__(16) uint32_t gcnt[];  // [B][32]
   pdl_trigger();
-  const uint32_t row = blockIdx.y, tid = threadIdx.x, lane = tid & 31;
+  const uint32_t row = blockIdx.z * kGenericGridRows + blockIdx.y, slice = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
+  if (row >= segs.rows) return;
   uint32_t seg = 0;
   while (seg + 1 < segs.count && row >= segs.s[seg + 1].row0) ++seg;
   const uint8_t* frame = segs.s[seg].frames + static_cast<uint64_t>(row - segs.s[seg].row0) * a.frame_bytes;
@@ -393,7 +402,7 @@ __global__ void __launch_bounds__(kGenericThreads) hist_generic_kernel(SegTable 
     const uint32_t mis = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(frame) & 15u);
     p_a = min(((16u - mis) * 11u) & 15u, npix);
     G = (npix - p_a) / 16;
-    g0 = blockIdx.x * a.slice_groups;
+    g0 = slice * a.slice_groups;
     g1 = min(g0 + a.slice_groups, G);
     base = frame + 3ull * p_a;
   };
@@ -409,7 +418,7 @@ __global__ void __launch_bounds__(kGenericThreads) hist_generic_kernel(SegTable 
   __syncthreads();
   const uint32_t cnt_lane = static_cast<uint32_t>(__cvta_generic_to_shared(gcnt)) + lane * 4;
   if (!kAhead) place();
-#pragma unroll 2
+#pragma unroll(kAhead ? 1 : 2)
   for (uint32_t g = g0 + tid; g < g1; g += kGenericThreads) {
     const uint4* p = reinterpret_cast<const uint4*>(base + 48ull * g);
     const uint4 x = __ldcs(p), y = __ldcs(p + 1), z = __ldcs(p + 2);
@@ -431,9 +440,9 @@ __global__ void __launch_bounds__(kGenericThreads) hist_generic_kernel(SegTable 
     const uint32_t b = generic_bin<kBin>(v, L);
     if (COFIE_BOUND(b < L.bins)) red_add_shared(cnt_lane + (b << 7));
   };
-  if (blockIdx.x == 0)
+  if (slice == 0)
     for (uint32_t q = tid; q < p_a; q += kGenericThreads) scalar(q);
-  if (blockIdx.x == gridDim.x - 1)
+  if (slice == gridDim.x - 1)
     for (uint32_t q = p_a + 16 * G + tid; q < npix; q += kGenericThreads) scalar(q);
   __syncthreads();
   for (uint32_t b = tid; b < L.bins; b += kGenericThreads) {
@@ -446,45 +455,30 @@ __global__ void __launch_bounds__(kGenericThreads) hist_generic_kernel(SegTable 
 
 }  // namespace
 
-static size_t hist_smem_bytes(uint32_t bins, int stages) {
-  return static_cast<size_t>(stages) * kChunkBytes + static_cast<size_t>(bins) * 32 * 4 + 2 * stages * 8;
+static size_t hist_smem_bytes(uint32_t bins) {
+  constexpr int kS = Shape<kBinFast>::stages;
+  return static_cast<size_t>(kS) * kChunkBytes + static_cast<size_t>(bins) * 32 * 4 + 2 * kS * 8;
 }
 
 static size_t cells_smem_bytes() {
-  return static_cast<size_t>(kCellStages) * kChunkBytes + static_cast<size_t>(kMaxBins) * 4 + 2 * kCellStages * 8;
+  constexpr int kS = Shape<kCells>::stages;
+  return static_cast<size_t>(kS) * kChunkBytes + static_cast<size_t>(kMaxBins) * 4 + 2 * kS * 8;
 }
 
-static auto hist_fast_variant(int bin_path, int stages) {
-  return bin_path == kBinFast
-             ? (stages == kStages ? hist_fast_kernel<kBinFast, kStages> : hist_fast_kernel<kBinFast, kStagesWide>)
-             : (stages == kStages ? hist_fast_kernel<kBinTwoStep, kStages> : hist_fast_kernel<kBinTwoStep, kStagesWide>);
-}
-
-// CTAs of the variant resident on an SM, or -1 on error.
-static int hist_occupancy(int bin_path, uint32_t bins, int stages) {
-  const auto kernel = hist_fast_variant(bin_path, stages);
-  const int limit = static_cast<int>(hist_smem_bytes(kMaxBins, stages));  // for every handle's bins: the limit is the kernel's
+int hist_blocks_per_sm(int bin_path, uint32_t bins) {
+  const auto kernel = bin_path == kBinFast ? hist_fast_kernel<kBinFast> : hist_fast_kernel<kBinTwoStep>;
+  const int limit = static_cast<int>(hist_smem_bytes(kMaxBins));  // for every handle's bins: the limit is the kernel's
   int n = 0;
   if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, limit) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, kThreads, hist_smem_bytes(bins, stages)) != cudaSuccess)
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, kThreads, hist_smem_bytes(bins)) != cudaSuccess)
     return -1;
   return n;
-}
-
-int hist_blocks_per_sm(int bin_path, uint32_t bins, int* stages) {
-  *stages = kStages;
-  const int n = hist_occupancy(bin_path, bins, kStages);
-  if (n != 1) return n;
-  const int wide = hist_occupancy(bin_path, bins, kStagesWide);
-  if (wide < 2) return n;
-  *stages = kStagesWide;
-  return wide;
 }
 
 uint32_t hist_chunk_groups() { return kChunkGroups; }
 
 int cells_blocks_per_sm() {
-  const auto kernel = hist_fast_kernel<kCells, kCellStages>;
+  const auto kernel = hist_fast_kernel<kCells>;
   const size_t smem = cells_smem_bytes();
   if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
     return -1;
@@ -494,22 +488,22 @@ int cells_blocks_per_sm() {
 
 cudaError_t launch_cells_fast(const SegTable& segs, const HistArgs& a, const LumaConsts& lc, uint32_t* cells,
                               uint32_t* err, int grid, cudaStream_t st, bool pdl) {
-  const cudaError_t e = launch_dependent(pdl, hist_fast_kernel<kCells, kCellStages>, dim3(grid),
+  const cudaError_t e = launch_dependent(pdl, hist_fast_kernel<kCells>, dim3(grid),
                                          dim3(Shape<kCells>::threads), cells_smem_bytes(), st, segs, a, lc, cells, err);
   return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
-cudaError_t launch_hist_fast(const SegTable& segs, const HistArgs& a, const LumaConsts& lc, int bin_path, int stages,
+cudaError_t launch_hist_fast(const SegTable& segs, const HistArgs& a, const LumaConsts& lc, int bin_path,
                              uint32_t* hist, uint32_t* err, int grid, cudaStream_t st, bool pdl) {
-  const cudaError_t e = launch_dependent(pdl, hist_fast_variant(bin_path, stages), dim3(grid), dim3(kThreads),
-                                         hist_smem_bytes(lc.bins, stages), st, segs, a, lc, hist, err);
+  const auto kernel = bin_path == kBinFast ? hist_fast_kernel<kBinFast> : hist_fast_kernel<kBinTwoStep>;
+  const cudaError_t e = launch_dependent(pdl, kernel, dim3(grid), dim3(kThreads), hist_smem_bytes(lc.bins), st, segs, a,
+                                         lc, hist, err);
   return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
 uint32_t hist_generic_slices(uint32_t npix, uint32_t slice_groups) {
-  const uint32_t spc = slice_groups ? slice_groups : kGenericGroupsPerCta;
   const uint32_t groups = npix / 16;  // at least the interior's groups, whatever the alignment
-  return groups ? (groups + spc - 1) / spc : 1;
+  return groups ? (groups + slice_groups - 1) / slice_groups : 1;
 }
 
 static auto hist_generic_variant(int bin_path, bool ahead) {
@@ -530,8 +524,11 @@ int hist_generic_blocks_per_sm(int bin_path, uint32_t bins) {
 cudaError_t launch_hist_generic(const SegTable& segs, const HistArgs& a, const LumaConsts& lc, int bin_path,
                                 uint32_t* hist, cudaStream_t st, uint32_t slice_groups, bool pdl) {
   HistArgs b = a;
-  b.slice_groups = slice_groups ? slice_groups : kGenericGroupsPerCta;
-  const dim3 grid(hist_generic_slices(a.npix, b.slice_groups), segs.rows);
+  // even slices of whole passes of a CTA's threads, at most as long as asked for
+  const uint32_t n = hist_generic_slices(a.npix, slice_groups), per = (a.npix / 16 + n - 1) / n;
+  b.slice_groups = std::max(1u, (per + kGenericThreads - 1) / kGenericThreads) * kGenericThreads;
+  const dim3 grid(hist_generic_slices(a.npix, b.slice_groups), std::min(segs.rows, kGenericGridRows),
+                  (segs.rows + kGenericGridRows - 1) / kGenericGridRows);
   const size_t smem = static_cast<size_t>(lc.bins) * 32 * 4;
   const cudaError_t e = launch_dependent(pdl, hist_generic_variant(bin_path, pdl), grid, dim3(kGenericThreads), smem, st, segs, b, lc, hist);
   return e == cudaSuccess ? cudaGetLastError() : e;
