@@ -24,6 +24,14 @@ def library_path() -> str:
     return _abi.LIB_PATH
 
 
+# The current CUDA stream's handle. torch's own accessor for it takes 0.1 us
+# against 1.9 us for building a Stream object; a push costs the host 10 us.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+if _raw_stream is None:
+    def _raw_stream(index):
+        return torch.cuda.current_stream(index).cuda_stream
+
+
 def _ptr(x) -> int | None:
     if x is None:
         return None
@@ -77,7 +85,7 @@ class NGFF:
 
     def _stream(self, cuda_stream):
         if cuda_stream is None:
-            return torch.cuda.current_stream(self.device).cuda_stream
+            return _raw_stream(self.device.index)
         if isinstance(cuda_stream, torch.cuda.Stream):
             return cuda_stream.cuda_stream
         return int(cuda_stream)
@@ -108,7 +116,8 @@ class NGFF:
         """Decides the next n frames of ``stream``; returns (scores, keep) or
         (scores, keep, hist). Asynchronous on the current CUDA stream."""
         n = self._frames(frames)
-        scores, keep, hist = self._outputs(frames, n, scores, keep, hist, return_hist or hist is not None)
+        if scores is None or keep is None or (hist is None and return_hist):
+            scores, keep, hist = self._outputs(frames, n, scores, keep, hist, return_hist)
         st = self._stream(cuda_stream)
         if hist is None:
             rc = self._lib.cofie_ngff_push(self._h, stream, _ptr(frames), n, _ptr(scores), _ptr(keep), st)
@@ -298,7 +307,7 @@ class QER:
         w = torch.empty(n, dtype=torch.float32, device=self.device)
         sel = torch.empty(n, dtype=torch.int32, device=self.device)
         kk = ctypes.c_uint32(0)
-        st = torch.cuda.current_stream(self.device).cuda_stream if cuda_stream is None else int(cuda_stream)
+        st = _raw_stream(self.device.index) if cuda_stream is None else int(cuda_stream)
         self._check(self._lib.cofie_qer_run(self._h, _ptr(q), _ptr(k), n, _ptr(w), _ptr(sel),
                                             ctypes.addressof(kk), st))
         return w, sel[: kk.value]
@@ -309,11 +318,11 @@ class QER:
         w [n_frames] float32, sel [n_frames] int32 (first k_dev[0] entries valid)."""
         T = self.params.tokens_per_frame
         n = k.shape[0] // T if n_frames is None else n_frames
-        st = torch.cuda.current_stream(self.device).cuda_stream if cuda_stream is None else int(cuda_stream)
+        st = _raw_stream(self.device.index) if cuda_stream is None else int(cuda_stream)
         self._check(self._lib.cofie_qer_run(self._h, _ptr(q), _ptr(k), n, _ptr(w), _ptr(sel), _ptr(k_dev), st))
 
     def status(self, cuda_stream=None):
-        st = torch.cuda.current_stream(self.device).cuda_stream if cuda_stream is None else int(cuda_stream)
+        st = _raw_stream(self.device.index) if cuda_stream is None else int(cuda_stream)
         self._check(self._lib.cofie_qer_status(self._h, st))
 
     def profile_reset(self, time_kernels: bool = False):

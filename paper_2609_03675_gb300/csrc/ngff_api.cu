@@ -84,7 +84,11 @@ struct cofie_ngff {
   float* d_scores = nullptr;
   uint8_t* d_keep = nullptr;
   uint32_t* d_err = nullptr;
-  uint32_t* d_count = nullptr;  // candidate count when the caller's m_out is host memory
+  // the candidate count when the caller's m_out is host memory: a word of
+  // mapped host memory that the kernel writes (a copy into pageable memory
+  // after the kernel costs the host 8 us of a 25 us call)
+  uint32_t* host_count = nullptr;
+  uint32_t* host_count_dev = nullptr;
   uint32_t* d_idx = nullptr;    // candidate indices when the caller's idx_out is host memory (allocated on first use)
   uint64_t dirty_rows = 0;      // histogram rows [0, dirty_rows) may be nonzero
   uint16_t* d_map = nullptr;    // a shard's gap map
@@ -616,8 +620,9 @@ void free_handle(cofie_ngff* h) {
   if (!h) return;
   DeviceGuard guard(h->device);
   cudaDeviceSynchronize();
+  if (h->host_count) cudaFreeHost(h->host_count);
   void* bufs[] = {h->d_hist,     h->d_l1,       h->d_mask,  h->d_ring, h->d_state, h->d_scores, h->d_keep,
-                  h->d_err,      h->d_stage[0], h->d_stage[1], h->d_count, h->d_map, h->d_cells, h->d_record, h->d_idx,
+                  h->d_err,      h->d_stage[0], h->d_stage[1], h->d_map, h->d_cells, h->d_record, h->d_idx,
                   h->d_chain_maps, h->d_chain_flags, h->d_lazy};
   for (void* b : bufs)
     if (b) cudaFree(b);
@@ -775,7 +780,8 @@ int cofie_ngff_create(const cofie_ngff_params* p, cofie_ngff_t** out) {
   if (e == cudaSuccess) e = dalloc(&h->d_scores, F);
   if (e == cudaSuccess) e = dalloc(&h->d_keep, F);
   if (e == cudaSuccess) e = dalloc(&h->d_err, 1);
-  if (e == cudaSuccess) e = dalloc(&h->d_count, 1);
+  if (e == cudaSuccess) e = cudaHostAlloc(reinterpret_cast<void**>(&h->host_count), sizeof(uint32_t), cudaHostAllocMapped);
+  if (e == cudaSuccess) e = cudaHostGetDevicePointer(reinterpret_cast<void**>(&h->host_count_dev), h->host_count, 0);
   if (e == cudaSuccess) e = dalloc(&h->d_map, COFIE_NGFF_MAX_LMAX);
   if (e == cudaSuccess) e = dalloc(&h->d_record, S * h->rec_words);
   const bool chained = p->l_max > 0 && p->signal != COFIE_SIGNAL_SCD;
@@ -1277,14 +1283,14 @@ int cofie_ngff_candidates(cofie_ngff_t* h, uint32_t stream, uint32_t* idx_out, u
     idx = h->d_idx;
     if (cap > h->p.max_stream_frames) cap = h->p.max_stream_frames;  // |S_c| <= T <= the record's frames
   }
-  uint32_t* count = km == kDevice ? m_out : h->d_count;
+  uint32_t* count = km == kDevice ? m_out : h->host_count_dev;
   cudaError_t e = launch_stream_candidates(h->d_record + static_cast<size_t>(stream) * h->rec_words, h->rec_words,
                                            h->d_state + stream, h->p.m_min, idx, cap, count, h->d_err, st);
   if (e != cudaSuccess) return h->cuda_fail(e, "candidates kernel launch");
   h->n_other += 1;
   if (km != kDevice) {
-    e = cudaMemcpyAsync(m_out, count, sizeof(uint32_t), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    e = cudaStreamSynchronize(st);
+    if (e == cudaSuccess) *m_out = *static_cast<volatile uint32_t*>(h->host_count);
     if (e == cudaSuccess && idx != idx_out && *m_out > 0)
       e = cudaMemcpy(idx_out, idx, static_cast<size_t>(std::min(*m_out, cap)) * sizeof(uint32_t),
                      cudaMemcpyDeviceToHost);
@@ -1313,13 +1319,13 @@ int cofie_ngff_candidates_from_keep(cofie_ngff_t* h, const uint8_t* keep, uint32
   if (!keep || !idx_out || classify(keep, &dk) != kDevice || classify(idx_out, &di) != kDevice || dk != h->device ||
       di != h->device)
     return h->fail(COFIE_EINVAL, "keep and idx_out must be device memory on the handle's device");
-  uint32_t* count = km == kDevice ? m_out : h->d_count;
+  uint32_t* count = km == kDevice ? m_out : h->host_count_dev;
   cudaError_t e = launch_candidates(keep, T, h->p.m_min, idx_out, count, st);
   if (e != cudaSuccess) return h->cuda_fail(e, "candidates kernel launch");
   h->n_other += 1;
   if (km != kDevice) {
-    e = cudaMemcpyAsync(m_out, count, sizeof(uint32_t), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    e = cudaStreamSynchronize(st);
+    if (e == cudaSuccess) *m_out = *static_cast<volatile uint32_t*>(h->host_count);
     if (e != cudaSuccess) return h->cuda_fail(e, "candidates count");
   }
   return COFIE_OK;

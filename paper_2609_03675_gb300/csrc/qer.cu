@@ -1009,7 +1009,8 @@ struct cofie_qer {
   float* d_colmax = nullptr;
   float* d_w = nullptr;
   uint8_t* d_flag = nullptr;
-  uint32_t* d_k = nullptr;
+  uint32_t* host_k = nullptr;  // the count when the caller's k_out is host memory: mapped, written by the kernel
+  uint32_t* host_k_dev = nullptr;
   uint32_t* d_done = nullptr;  // CTAs of the ranking kernel that have finished
   uint32_t* d_err = nullptr;
   std::string err;
@@ -1042,7 +1043,8 @@ void qer_free(cofie_qer* h) {
   cudaGetDevice(&prev);
   cudaSetDevice(h->device);
   cudaDeviceSynchronize();
-  void* bufs[] = {h->d_qg, h->d_colmax, h->d_w, h->d_k, h->d_err, h->d_flag, h->d_done};
+  if (h->host_k) cudaFreeHost(h->host_k);
+  void* bufs[] = {h->d_qg, h->d_colmax, h->d_w, h->d_err, h->d_flag, h->d_done};
   for (void* b : bufs)
     if (b) cudaFree(b);
   for (cudaEvent_t e : h->ev) cudaEventDestroy(e);
@@ -1110,7 +1112,8 @@ int cofie_qer_create(const cofie_qer_params* p, cofie_qer_t** out) {
   cudaError_t e = cudaMalloc(&h->d_qg, static_cast<size_t>(h->n_blk) * h->n_pad * D * 2);
   if (e == cudaSuccess) e = cudaMalloc(&h->d_colmax, nv * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc(&h->d_w, static_cast<size_t>(p->max_frames) * sizeof(float));
-  if (e == cudaSuccess) e = cudaMalloc(&h->d_k, sizeof(uint32_t));
+  if (e == cudaSuccess) e = cudaHostAlloc(reinterpret_cast<void**>(&h->host_k), sizeof(uint32_t), cudaHostAllocMapped);
+  if (e == cudaSuccess) e = cudaHostGetDevicePointer(reinterpret_cast<void**>(&h->host_k_dev), h->host_k, 0);
   if (e == cudaSuccess) e = cudaMalloc(&h->d_flag, p->max_frames);
   if (e == cudaSuccess) e = cudaMalloc(&h->d_done, sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMemset(h->d_done, 0, sizeof(uint32_t));
@@ -1239,7 +1242,7 @@ int cofie_qer_run(cofie_qer_t* h, const uint16_t* q, const uint16_t* k, uint32_t
   const uint32_t kk = static_cast<uint32_t>(std::max(1.0, std::nearbyint(static_cast<double>(p.rho) * n_frames)));
   const float scale = static_cast<float>(1.0 / (static_cast<double>(p.n_heads) * std::sqrt(static_cast<double>(p.head_dim))));
   float* w = w_out ? w_out : h->d_w;
-  uint32_t* kdev = is_device(k_out, h->device) ? k_out : h->d_k;
+  uint32_t* kdev = is_device(k_out, h->device) ? k_out : h->host_k_dev;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (h->time_on && !capturing && h->ev_used + 2 <= (1u << 16)) {
     while (h->ev.size() < h->ev_used + 2) {
@@ -1325,8 +1328,8 @@ int cofie_qer_run(cofie_qer_t* h, const uint16_t* q, const uint16_t* k, uint32_t
   }
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess && kdev != k_out) {
-    e = cudaMemcpyAsync(k_out, kdev, sizeof(uint32_t), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    e = cudaStreamSynchronize(st);
+    if (e == cudaSuccess) *k_out = *static_cast<volatile uint32_t*>(h->host_k);
   }
   if (e != cudaSuccess) return h->fail(COFIE_ECUDA, std::string("QER launch: ") + cudaGetErrorString(e));
   return COFIE_OK;
