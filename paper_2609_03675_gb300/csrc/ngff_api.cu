@@ -69,6 +69,7 @@ struct cofie_ngff {
   bool size_fast = false;
   int hist_grid = 0;
   uint64_t generic_wave = 0;  // CTAs of the generic kernel resident at once
+  int span_grid = 0;          // CTAs of the even-share kernel resident at once
   int cells_grid = 0;    // the TMA kernel's grid for the spatial signals (0: not usable)
   unsigned long long x_tau = 0, x_cut = 0, x_grad = 0;  // integer forms of the fp32 decisions
   uint32_t m_gpr = 0, m_h = 0, m_gw = 0;  // its multiply-high divisors (16-pixel groups per row, height, grid columns)
@@ -344,11 +345,14 @@ cudaError_t launch_first_stage(cofie_ngff* h, const SegTable& segs, cudaStream_t
   //    12.4; one 4K frame 10.8 on K1, 8.7; 60 frames 19.6 with kWaveGroups,
   //    18.3); with many bins to clear and fold 512 from 480,000 groups on (40
   //    frames, 128 bins: 21.3 on kWaveGroups, 20.5 with 256, 19.6 with 512);
-  //  - up to one resident wave and an eighth of a second: kWaveGroups, as an
-  //    ordinary launch, whose CTAs start as SMs free (serving calls of 133
-  //    frames of 640x360: 24.3 us against 25.0 with half of that, 30.2 with
-  //    256 groups; made resident ahead of time they crowd the SMs that the
-  //    kernel before still holds);
+  //  - up to one resident wave and an eighth of a second: aligned frames of at
+  //    least kWaveGroups in even shares, from 1,750,000 groups on (serving
+  //    calls of 133 frames of 640x360 21.7 us, 20 1080p frames from a graph 25.9
+  //    against 29.4; but 110 frames of 640x360 21.7 against 21.0); others in
+  //    slices of kWaveGroups, as an ordinary launch, whose
+  //    CTAs start as SMs free (the same calls 24.1 us, 25.0 with half of that,
+  //    30.2 with 256 groups; made resident ahead of time they crowd the SMs
+  //    that the kernel before still holds);
   //  - larger: slices short enough that the last wave's share is small, longer
   //    with many bins (220 frames of 640x360: 105.7 on K1, 100.8 with 512, 104
   //    with 1024; 600 1080p frames: 517 on K1, 544 with 512, 509 with 1024, 511
@@ -367,6 +371,8 @@ cudaError_t launch_first_stage(cofie_ngff* h, const SegTable& segs, cudaStream_t
     const uint64_t groups = static_cast<uint64_t>(h->npix / 16) * segs.rows;
     const uint32_t longer = h->lc.bins > 128 ? 2 : (h->lc.bins > 64 ? 1 : 0);
     if (wave_ctas < 5 * sms) return generic(longer && groups >= 480000 ? 512 : 256, pdl);
+    if (wave_ctas <= hi && fast && groups >= 1750000 && ha.groups_per_frame >= kWaveGroups)
+      return launch_hist_span(segs, ha, h->lc, h->bin_path, h->d_hist, h->span_grid, st, pdl);
     if (wave_ctas <= hi) return generic(kWaveGroups, false);
     return generic((groups < 4000000 ? 512u : 1024u) << longer, false);
   }
@@ -816,6 +822,9 @@ int cofie_ngff_create(const cofie_ngff_params* p, cofie_ngff_t** out) {
     const int per_sm = hist_blocks_per_sm(h->bin_path, p->bins);
     if (per_sm <= 0) e = cudaGetLastError() != cudaSuccess ? cudaErrorInvalidConfiguration : cudaErrorInvalidValue;
     h->hist_grid = h->num_sms * (per_sm > 0 ? per_sm : 1);
+    const int span_per_sm = hist_span_blocks_per_sm(h->bin_path, p->bins);
+    if (span_per_sm <= 0) e = cudaErrorInvalidConfiguration;
+    h->span_grid = h->num_sms * (span_per_sm > 0 ? span_per_sm : 1);
   }
   if (e == cudaSuccess) {
     const int gen_per_sm = hist_generic_blocks_per_sm(h->bin_path, p->bins);

@@ -51,3 +51,32 @@ def test_more_rows_than_a_grid_dimension():
     f.status()
     assert np.array_equal(k.cpu().numpy(), ko)
     assert np.all(np.abs(s.cpu().numpy().astype(np.float64) - so) <= 1e-6 * so)
+
+
+@pytest.mark.parametrize("w,h,counts", [(640, 360, [1, 0, 30, 8, 91]), (640, 360, [18] * 9), (224, 224, [97, 500, 13]),
+                                        (1920, 1080, [2, 7, 6])])
+@pytest.mark.parametrize("bins", [32, 48, 128])
+def test_even_shares_over_segments(w, h, counts, bins):
+    """Batched calls of about one resident wave: shares that end inside frames
+    and pass from one stream's frames to the next stream's, in other memory."""
+    from paper_2609_03675_gb300 import NGFF
+    rng = np.random.default_rng(sum(counts) + bins)
+    base = rng.integers(0, 256, (5, h, w, 3), dtype=np.uint8)
+    base[4] = 255
+    p = O.Params(w, h, bins=bins, tau=0.02)
+    f = NGFF(w, h, bins=bins, tau=0.02, max_streams=len(counts))
+    src = torch.from_numpy(base).cuda()
+    items, picks = [], []
+    for s, n in enumerate(counts):
+        pick = rng.integers(0, 5, n)
+        picks.append(pick)
+        items.append((s, src[torch.from_numpy(pick).cuda()], torch.empty(n, device="cuda"),
+                      torch.empty(n, dtype=torch.uint8, device="cuda")))
+    f.push_batch(items)
+    torch.cuda.synchronize()
+    f.status()
+    for (s, _, sc, kp), pick in zip(items, picks):
+        if len(pick):
+            _, so, ko = O.load().run(base[pick], p)
+            assert np.array_equal(kp.cpu().numpy(), ko), s
+            assert np.all(np.abs(sc.cpu().numpy().astype(np.float64) - so) <= 1e-6 * so), s
