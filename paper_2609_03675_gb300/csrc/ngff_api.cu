@@ -458,7 +458,7 @@ int run_segments(cofie_ngff* h, const SegTable& segs, cudaStream_t st, bool keep
   // pushes clear their rows inside the selection kernel (saving a launch),
   // except where the window and scan kernels or the larger selection without
   // forced retention decide them: there one memset after the selection does
-  const bool walk = h->p.l_max > 0 && h->p.l_max <= select_walk_max_lmax() && longest <= select_walk_max_frames();
+  const bool walk = select_walk_takes(longest, sa);
   const bool chain = h->p.l_max > 0 && !walk && !sa.scd;
   const bool fused = longest <= select_small_max();
   const bool lazy_walk = h->p.l_max == 0 && lazy_walk_fits(longest, h->fw);

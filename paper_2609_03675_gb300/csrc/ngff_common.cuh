@@ -268,9 +268,8 @@ cudaError_t launch_scan(const SegTable& segs, const SelectArgs& a, const uint32_
 uint32_t select_small_max();
 cudaError_t launch_select_small(const SegTable& segs, const SelectArgs& a, uint32_t* hist, uint32_t* ring,
                                 StreamState* state, uint32_t* l1, uint32_t* mask, cudaStream_t st, bool pdl = false);
-// pushes of at most select_walk_max_frames() frames per stream with L_max <= select_walk_max_lmax()
-uint32_t select_walk_max_frames();
-uint32_t select_walk_max_lmax();
+// whether one CTA per stream walks the rule of a push whose longest piece of a stream is `longest`
+bool select_walk_takes(uint32_t longest, const SelectArgs& a);
 cudaError_t launch_select_walk(const SegTable& segs, const SelectArgs& a, uint32_t* hist, uint32_t* ring,
                                StreamState* state, cudaStream_t st, bool pdl = false);
 cudaError_t launch_cells_any(const SegTable& segs, const FeatArgs& fa, const LumaConsts& lc, uint32_t* cells,

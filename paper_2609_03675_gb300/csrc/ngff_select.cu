@@ -45,7 +45,7 @@ constexpr uint32_t kSmallMax = 64;    // frames per stream segment for the fused
 constexpr int kWalkThreads = 256;
 constexpr uint32_t kWalkMaxFrames = 64;
 constexpr uint32_t kWalkMaxLmax = 64;
-constexpr size_t kWalkStageBudget = 48 * 1024;  // shared memory a walk CTA takes without opting in
+constexpr size_t kWalkSmemMax = 160 * 1024;  // 64 frames, L_max = 64, 256 words a row: 148 KiB
 
 __device__ __forceinline__ uint32_t absdiff(uint32_t a, uint32_t b) { return a > b ? a - b : b - a; }
 
@@ -385,10 +385,10 @@ __global__ void __launch_bounds__(kScanThreads) select_small_kernel(SegTable seg
 
 // Small pushes, one 256-thread CTA per stream segment (n <= kWalkMaxFrames,
 // L_max <= kWalkMaxLmax), in the order the rule states it:
-//   0. (kStaged) the stream's ring of the last L_max rows and the push's own
-//      rows are copied into shared memory in one coalesced pass, alongside
-//      the read of the stream's state, so that everything after it reads
-//      shared memory only;
+//   0. the stream's ring of the last L_max rows and the push's own rows are
+//      copied into shared memory in one coalesced pass, alongside the read of
+//      the stream's state, so that everything after it reads shared memory
+//      only;
 //   1. windowed distances, a warp per frame, lane = lag k (the Eq. 2
 //      numerators L1[j][k-1] = sum_b |c_t - c_{t-k}|), each lane starting at
 //      a column rotated by its lane so a warp's 16-byte reads of different
@@ -403,9 +403,7 @@ __global__ void __launch_bounds__(kScanThreads) select_small_kernel(SegTable seg
 //   3. all threads emit scores and keep codes, note retained frames in the
 //      stream's retention record, store the last L_max rows in the ring,
 //      update the stream state and zero the push's rows for the next push.
-// Without kStaged (rows too wide for the staging budget) the same steps read
-// the rows from global memory.
-template <bool kVec4, bool kStaged>
+template <bool kVec4>
 __global__ void __launch_bounds__(kWalkThreads) select_walk_kernel(SegTable segs, SelectArgs a,
                                                                    uint32_t* __restrict__ hist,
                                                                    uint32_t* __restrict__ ring,
@@ -421,8 +419,8 @@ __global__ void __launch_bounds__(kWalkThreads) select_walk_kernel(SegTable segs
   const uint32_t n = sg.n, row0 = sg.row0, stream = sg.stream;
   const uint32_t B = a.bins, L = a.l_max, W = a.mask_words;
   if (n == 0) return;
-  uint32_t* srows = wsm;                                   // kStaged: [L + n][B], ring slots then the push
-  uint32_t* sl1 = wsm + (kStaged ? (L + n) * B : 0u);      // [n][L]
+  uint32_t* srows = wsm;                                   // [L + n][B], ring slots then the push
+  uint32_t* sl1 = wsm + (L + n) * B;                       // [n][L]
   uint32_t* smask = sl1 + n * L;                           // [n][W]
   uint32_t* sgap = smask + n * W;                          // [n]: gap, bit 31 a scene change
   const uint32_t* ring_s = ring + static_cast<uint64_t>(stream) * L * B;
@@ -433,37 +431,34 @@ __global__ void __launch_bounds__(kWalkThreads) select_walk_kernel(SegTable segs
     s_g = state[stream].g;
     s_slot0 = static_cast<uint32_t>(s_t0 % L);  // the ring slot of the push's first frame (one 64-bit division)
   }
-  if (kStaged) {
-    if (kVec4) {
-      const uint32_t rq = L * B / 4, hq = n * B / 4;
-      for (uint32_t i = tid; i < rq + hq; i += kWalkThreads)
-        reinterpret_cast<uint4*>(srows)[i] =
-            i < rq ? reinterpret_cast<const uint4*>(ring_s)[i] : reinterpret_cast<const uint4*>(hist_s)[i - rq];
-    } else {
-      for (uint32_t i = tid; i < (L + n) * B; i += kWalkThreads)
-        srows[i] = i < L * B ? ring_s[i] : hist_s[i - L * B];
-    }
+  if (kVec4) {
+    const uint32_t rq = L * B / 4, hq = n * B / 4;
+    for (uint32_t i = tid; i < rq + hq; i += kWalkThreads)
+      reinterpret_cast<uint4*>(srows)[i] =
+          i < rq ? reinterpret_cast<const uint4*>(ring_s)[i] : reinterpret_cast<const uint4*>(hist_s)[i - rq];
+  } else {
+    for (uint32_t i = tid; i < (L + n) * B; i += kWalkThreads) srows[i] = i < L * B ? ring_s[i] : hist_s[i - L * B];
   }
   __syncthreads();
   const unsigned long long t0 = s_t0;
   const int slot0 = static_cast<int>(s_slot0), Li = static_cast<int>(L);
-  const uint32_t nq = B / 4, rot = kStaged && kVec4 ? lane % max(nq, 1u) : 0u;
+  const uint32_t nq = B / 4, rot = kVec4 ? lane % max(nq, 1u) : 0u;
 
   // 1. distances and keep bits
   for (uint32_t j = warp; j < n; j += kWarps) {
     const unsigned long long t = t0 + j;
-    const uint32_t* ct = kStaged ? srows + (L + j) * B : hist_s + static_cast<uint64_t>(j) * B;
+    const uint32_t* ct = srows + (L + j) * B;
     uint32_t l_adj = 0;
     for (uint32_t w = 0; w < W; ++w) {
       const uint32_t k = 32 * w + lane + 1;
       const bool valid = k <= L && k <= t;
       const uint32_t* src = ct;
       if (valid) {
-        if (k <= j) src = ct - static_cast<uint64_t>(k) * B;
+        if (k <= j) src = ct - k * B;
         else {  // ring slot of frame t - k: (slot0 + j - k) mod L, with |j - k| < 2^7
           int slot = (slot0 + static_cast<int>(j) - static_cast<int>(k)) % Li;
           if (slot < 0) slot += Li;
-          src = (kStaged ? srows : ring_s) + static_cast<uint32_t>(slot) * B;
+          src = srows + static_cast<uint32_t>(slot) * B;
         }
       }
       uint32_t d = 0;
@@ -554,7 +549,7 @@ __global__ void __launch_bounds__(kWalkThreads) select_walk_kernel(SegTable segs
   uint32_t* ring_w = ring + static_cast<uint64_t>(stream) * L * B;
   for (uint32_t i = tid; i < keep_n * B; i += kWalkThreads) {
     const uint32_t jj = n - keep_n + i / B, b = i % B;
-    ring_w[((s_slot0 + jj) % L) * B + b] = kStaged ? srows[(L + jj) * B + b] : hist_s[static_cast<uint64_t>(jj) * B + b];
+    ring_w[((s_slot0 + jj) % L) * B + b] = srows[(L + jj) * B + b];
   }
   if (tid == 0) {
     state[stream].t = t0 + n;
@@ -562,13 +557,12 @@ __global__ void __launch_bounds__(kWalkThreads) select_walk_kernel(SegTable segs
     state[stream].acc = s_acc;
   }
   if (a.zero_hist) {
-    if (!kStaged) __syncthreads();  // the ring copies above have read the rows
     for (uint32_t i = tid; i < n * B; i += kWalkThreads) hist[static_cast<uint64_t>(row0) * B + i] = 0;
   }
 }
 
-size_t walk_smem_bytes(uint32_t n, uint32_t l_max, uint32_t mask_words, uint32_t bins, bool staged) {
-  return (static_cast<size_t>(n) * (l_max + mask_words + 1) + (staged ? static_cast<size_t>(l_max + n) * bins : 0)) * 4;
+size_t walk_smem_bytes(uint32_t n, uint32_t l_max, uint32_t mask_words, uint32_t bins) {
+  return (static_cast<size_t>(n) * (l_max + mask_words + 1) + static_cast<size_t>(l_max + n) * bins) * 4;
 }
 
 // The gap map of one stream segment: map[g-1] = the gap after its last frame
@@ -635,21 +629,25 @@ size_t scan_smem_bytes(uint32_t mask_words, uint32_t l_max) {
 }  // namespace
 
 uint32_t select_small_max() { return kSmallMax; }
-uint32_t select_walk_max_frames() { return kWalkMaxFrames; }
-uint32_t select_walk_max_lmax() { return kWalkMaxLmax; }
+// Wide rows (256 words past 15 frames at L_max = 30) are more than one CTA gets
+// through as fast as tiles over several do: pushes of 20 and 45 frames of
+// 640x360 with the low-res signal, from a graph, took 45 and 89 us when the walk
+// read their rows from global memory, 16 and 22 in tiles; 48 frames of 448x448
+// with 256 bins 84 and 21. Scene changes, which the tiles do not take, are
+// walked from shared memory whatever their size (those 48 frames: 86, now 35).
+bool select_walk_takes(uint32_t longest, const SelectArgs& a) {
+  return a.l_max > 0 && a.l_max <= kWalkMaxLmax && longest <= kWalkMaxFrames &&
+         (a.scd || walk_smem_bytes(longest, a.l_max, a.mask_words, a.bins) <= 48 * 1024);
+}
 
 cudaError_t launch_select_walk(const SegTable& segs, const SelectArgs& a, uint32_t* hist, uint32_t* ring,
                                StreamState* state, cudaStream_t st, bool pdl) {
   uint32_t longest = 0;
   for (uint32_t i = 0; i < segs.count; ++i) longest = max(longest, segs.s[i].n);
-  // rows staged in shared memory when they fit the default 48 KiB with the tables
-  const bool staged = walk_smem_bytes(longest, a.l_max, a.mask_words, a.bins, true) <= kWalkStageBudget;
-  const size_t smem = walk_smem_bytes(longest, a.l_max, a.mask_words, a.bins, staged);  // <= 48 KiB
+  const size_t smem = walk_smem_bytes(longest, a.l_max, a.mask_words, a.bins);
   const bool vec = a.bins % 4 == 0 && a.dist_kind == 0;
-  const auto kernel = vec ? (staged ? select_walk_kernel<true, true> : select_walk_kernel<true, false>)
-                          : (staged ? select_walk_kernel<false, true> : select_walk_kernel<false, false>);
-  const cudaError_t e =
-      launch_dependent(pdl, kernel, dim3(segs.count), dim3(kWalkThreads), smem, st, segs, a, hist, ring, state);
+  const cudaError_t e = launch_dependent(pdl, vec ? select_walk_kernel<true> : select_walk_kernel<false>, dim3(segs.count),
+                                         dim3(kWalkThreads), smem, st, segs, a, hist, ring, state);
   return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
@@ -676,7 +674,10 @@ cudaError_t launch_ring_store(const uint32_t* hist, uint32_t rows, unsigned long
 
 cudaError_t scan_prepare(uint32_t mask_words, uint32_t l_max) {
   const int smem = static_cast<int>(scan_smem_bytes(mask_words, l_max));
-  cudaError_t e;
+  cudaError_t e = cudaFuncSetAttribute(select_walk_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWalkSmemMax);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(select_walk_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWalkSmemMax);
+  if (e != cudaSuccess) return e;
   if (mask_words == 1) {
     e = cudaFuncSetAttribute(scan_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess)

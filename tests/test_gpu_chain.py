@@ -72,3 +72,27 @@ def test_batches_of_unequal_lengths(bins, l_max):
         _, so, ko = oracle_run(fr[s], O.Params(W, H, bins=bins, l_max=l_max, tau=tau))
         assert np.array_equal(outs[s][1].cpu().numpy(), ko), s
         assert np.all(np.abs(outs[s][0].cpu().numpy().astype(np.float64) - so) <= 1e-6 * so), s
+
+
+@pytest.mark.parametrize("bins,l_max", [(256, 30), (256, 64), (255, 30), (128, 33)])
+@pytest.mark.parametrize("scd", [False, True])
+def test_small_pushes_of_wide_rows(bins, l_max, scd):
+    """Pushes of up to 64 frames whose rows with the walk's tables are a little
+    under, at and over 48 KiB (15, 16 and 17 frames at 256 words, L_max = 30)."""
+    from oracle import scd_oracle as SC
+    from paper_2609_03675_gb300 import NGFF, _abi
+    sizes = [3, 15, 16, 17, 1, 33, 64, 63]
+    fr = _frames(sum(sizes), seed=61)
+    p = O.Params(W, H, bins=bins, l_max=l_max, tau=0.5)
+    kw = dict(bins=bins, l_max=l_max, tau=0.5)
+    if scd:
+        _, so, ko = SC.run(fr, p, 0.6, 0.2)
+        kw.update(signal=_abi.SIGNAL_SCD, scd_cut=0.6, scd_gradual=0.2)
+    else:
+        _, so, ko = oracle_run(fr, p)
+    f = NGFF(W, H, **kw)
+    got = [f.push(part) for part in torch.split(torch.from_numpy(fr).cuda(), sizes)]
+    torch.cuda.synchronize()
+    f.status()
+    assert np.array_equal(torch.cat([k for _, k in got]).cpu().numpy(), ko)
+    assert np.all(np.abs(torch.cat([s for s, _ in got]).cpu().numpy().astype(np.float64) - so) <= 1e-6 * so)
