@@ -318,7 +318,14 @@ cudaError_t launch_first_stage(cofie_ngff* h, const SegTable& segs, cudaStream_t
   if (cells) {
     const bool dhash = h->p.signal == COFIE_SIGNAL_DHASH;
     uint32_t* cells_out = dhash ? h->d_cells : h->d_hist;
-    if (!fast) {
+    // small launches run in slices, whose loads need no ring to fill: under
+    // 250,000 16-pixel groups (dHash from a graph: 10 frames of 640x360 8.4
+    // against 9.5 us, one 1080p frame 7.2 against 8.4; 20 frames 12.0 against
+    // 11.5), or 30,000 with cell columns under 16 pixels, which the slices take
+    // pixel by pixel (low-res, 224x224: 2 frames 7.8 against 9.8, 48 22.5
+    // against 18.1)
+    const bool wide_cells = h->p.width / h->fa.grid_w >= 16;
+    if (!fast || static_cast<uint64_t>(h->npix / 16) * segs.rows < (wide_cells ? 250000u : 30000u)) {
       cudaError_t e = launch_cells_any(segs, h->fa, h->lc, cells_out, h->num_sms, st, pdl);
       if (e == cudaSuccess && dhash) e = launch_dhash_finish(h->d_cells, segs.rows, h->fa, h->d_hist, st, true);
       return e;

@@ -223,6 +223,7 @@ struct FeatArgs {
   uint32_t use_magic;         // Y = umulhi(v, magic_y) (host-verified), else v / den
   uint32_t m_col;             // floor(2^32 grid_w / width), at most 2^32 - 1
   uint32_t slice_groups, slices;  // a launch's 16-pixel groups per CTA, and CTAs per frame
+  uint32_t ahead;                 // the launch is a programmatic dependent of the kernel before it
   uint32_t row_h[16], col_w[16];  // pixels per cell row / cell column
 };
 

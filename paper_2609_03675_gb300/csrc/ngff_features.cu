@@ -55,6 +55,16 @@ __global__ void __launch_bounds__(kAnyThreads, 6) cells_any_kernel(SegTable segs
   const uint32_t gh_shift = 31 - __clz(gh);  // 8 or 16 cell rows
   for (uint32_t i = tid; i < n_cells * kCellCopies; i += kAnyThreads) cell[i] = 0;
   if (tid <= gw) colstart[tid] = static_cast<uint32_t>((static_cast<uint64_t>(tid) * W + gw - 1) / gw);
+  // first 16-byte aligned pixel: 3 p = -(frame mod 16) mod 16, and 3 * 11 = 1 mod 16
+  const uint32_t mis = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(frame) & 15u);
+  const uint32_t p_a = min(((16u - mis) * 11u) & 15u, fa.npix);
+  const uint32_t G = (fa.npix - p_a) / 16;
+  const uint32_t g0 = slice * fa.slice_groups, g1 = min(g0 + fa.slice_groups, G);
+  const uint8_t* base = frame + 3ull * p_a;
+  // a programmatic dependent has its slice fetched into L2 while it waits (a
+  // hint, as in the generic histogram kernel)
+  if (fa.ahead && tid == 0 && g0 < g1)
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(base + 48ull * g0), "r"(48 * (g1 - g0)) : "memory");
   pdl_wait();  // no frame is read and no cell written before the kernel before this one has completed
   __syncthreads();
 
@@ -65,12 +75,6 @@ __global__ void __launch_bounds__(kAnyThreads, 6) cells_any_kernel(SegTable segs
   // first image row of the cell row after crow
   const auto next_cell_row = [&](uint32_t crow) { return ((crow + 1) * H + gh - 1) >> gh_shift; };
 
-  // first 16-byte aligned pixel: 3 p = -(frame mod 16) mod 16, and 3 * 11 = 1 mod 16
-  const uint32_t mis = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(frame) & 15u);
-  const uint32_t p_a = min(((16u - mis) * 11u) & 15u, fa.npix);
-  const uint32_t G = (fa.npix - p_a) / 16;
-  const uint32_t g0 = slice * fa.slice_groups, g1 = min(g0 + fa.slice_groups, G);
-  const uint8_t* base = frame + 3ull * p_a;
   if (g0 + tid < g1) {
     const uint32_t q = p_a + 16 * (g0 + tid);
     const uint32_t dr = 16 * kAnyThreads / W, dx = 16 * kAnyThreads - dr * W;
@@ -234,6 +238,7 @@ cudaError_t launch_cells_any(const SegTable& segs, const FeatArgs& fa, const Lum
   // a programmatic dependent only while its CTAs leave room on the SMs that
   // the kernel before it still holds (as the generic histogram kernel)
   pdl = pdl && ctas <= 4ull * num_sms;
+  f.ahead = pdl ? 1u : 0u;
   const auto kernel = fa.use_magic ? (wide ? cells_any_kernel<false, true> : cells_any_kernel<false, false>)
                                    : (wide ? cells_any_kernel<true, true> : cells_any_kernel<true, false>);
   const cudaError_t e = launch_dependent(pdl, kernel, dim3(static_cast<uint32_t>(ctas)), dim3(kAnyThreads), 0, st, segs,
