@@ -446,7 +446,10 @@ cudaError_t clear_rows(cofie_ngff* h, uint64_t rows, cudaStream_t st) {
 // prepared shard, a push that failed part way) are cleared first.
 // While `capturing`, nothing here runs until the graph is launched, so the
 // host's record of dirty rows is left as it was and no timing events are taken.
-int run_segments(cofie_ngff* h, const SegTable& segs, cudaStream_t st, bool keep_hist, bool capturing) {
+// keep_hist is cleared when the selection has written the rows to hist_out
+// itself (device memory of the handle's device, a push of one stream) and
+// zeroed them.
+int run_segments(cofie_ngff* h, const SegTable& segs, cudaStream_t st, bool* keep_hist, uint32_t* hist_out, bool capturing) {
   if (segs.rows == 0) return COFIE_OK;
   cudaError_t e = clear_rows(h, h->dirty_rows, st);
   if (e != cudaSuccess) return h->cuda_fail(e, "memset histograms");
@@ -469,7 +472,11 @@ int run_segments(cofie_ngff* h, const SegTable& segs, cudaStream_t st, bool keep
   const bool chain = h->p.l_max > 0 && !walk && !sa.scd;
   const bool fused = longest <= select_small_max();
   const bool lazy_walk = h->p.l_max == 0 && lazy_walk_fits(longest, h->fw);
-  sa.zero_hist = ((walk || chain || lazy_walk || (fused && h->p.l_max > 0)) && !keep_hist) ? 1u : 0u;
+  if (*keep_hist && hist_out && (walk || chain || lazy_walk)) {
+    sa.hist_out = hist_out;
+    *keep_hist = false;
+  }
+  sa.zero_hist = ((walk || chain || lazy_walk || (fused && h->p.l_max > 0)) && !*keep_hist) ? 1u : 0u;
   cudaEvent_t es0 = nullptr, es1 = nullptr;
   if (timed && take_pair(h->ev_sel, h->ev_sel_used, &es0, &es1)) cudaEventRecord(es0, st);
   if (lazy_walk) {  // no forced retention, few frames
@@ -502,7 +509,7 @@ int run_segments(cofie_ngff* h, const SegTable& segs, cudaStream_t st, bool keep
     h->n_select += 2;
   }
   if (es1) cudaEventRecord(es1, st);
-  if (keep_hist) {  // the caller clears the rows once it has copied them
+  if (*keep_hist) {  // the caller clears the rows once it has copied them
     if (!capturing) h->dirty_rows = segs.rows;
     return COFIE_OK;
   }
@@ -515,8 +522,9 @@ int run_segments(cofie_ngff* h, const SegTable& segs, cudaStream_t st, bool keep
 }
 
 // One piece of a single-stream push: n <= max_frames_per_push device frames.
+// hist_here: hist_out is memory of the handle's device.
 int run_piece(cofie_ngff* h, uint32_t stream, const uint8_t* dframes, uint32_t n, float* scores, MemKind ks,
-              uint8_t* keep, MemKind kk, uint32_t* hist_out, MemKind kh, cudaStream_t st, bool capturing) {
+              uint8_t* keep, MemKind kk, uint32_t* hist_out, MemKind kh, bool hist_here, cudaStream_t st, bool capturing) {
   SegTable segs;
   memset(&segs, 0, sizeof segs);
   segs.count = 1;
@@ -528,18 +536,19 @@ int run_piece(cofie_ngff* h, uint32_t stream, const uint8_t* dframes, uint32_t n
   s.stream = stream;
   s.scores = ks == kDevice ? scores : (ks == kNull ? nullptr : h->d_scores);
   s.keep = kk == kDevice ? keep : (kk == kNull ? nullptr : h->d_keep);
-  int rc = run_segments(h, segs, st, kh != kNull, capturing);
+  bool copy_hist = kh != kNull;  // the rows are left for a copy
+  int rc = run_segments(h, segs, st, &copy_hist, hist_here ? hist_out : nullptr, capturing);
   if (rc != COFIE_OK) return rc;
   cudaError_t e = cudaSuccess;
   if (ks == kHostPinned || ks == kHostPageable)
     e = cudaMemcpyAsync(scores, h->d_scores, n * sizeof(float), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess && (kk == kHostPinned || kk == kHostPageable))
     e = cudaMemcpyAsync(keep, h->d_keep, n, cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess && kh != kNull)
+  if (e == cudaSuccess && copy_hist)
     e = cudaMemcpyAsync(hist_out, h->d_hist, static_cast<size_t>(n) * h->fw * 4, cudaMemcpyDefault, st);
-  if (e == cudaSuccess && kh != kNull) e = clear_rows(h, n, st);
+  if (e == cudaSuccess && copy_hist) e = clear_rows(h, n, st);
   if (e != cudaSuccess) return h->cuda_fail(e, "output copy");
-  if (kh != kNull && !capturing) h->dirty_rows = 0;
+  if (copy_hist && !capturing) h->dirty_rows = 0;
   return COFIE_OK;
 }
 
@@ -583,7 +592,9 @@ int push_impl(cofie_ngff* h, uint32_t stream, const uint8_t* frames, uint32_t n,
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   int fdev = -1;
   const MemKind kf = classify(frames, &fdev);
-  const MemKind ks = classify(scores), kk = classify(keep), kh = classify(hist_out);
+  int hdev = -1;
+  const MemKind ks = classify(scores), kk = classify(keep), kh = classify(hist_out, &hdev);
+  const bool hist_here = kh == kDevice && hdev == h->device;
   if (kf == kDevice && fdev != h->device) return h->fail(COFIE_EINVAL, "frames live on another device");
   const int cap = capture_state(st);
   if (cap < 0) return h->fail(COFIE_ECUDA, "cannot read the CUDA stream's capture state");
@@ -598,7 +609,7 @@ int push_impl(cofie_ngff* h, uint32_t stream, const uint8_t* frames, uint32_t n,
       const uint32_t m = n - off < step ? n - off : step;
       int rc = run_piece(h, stream, frames + off * h->frame_bytes, m, scores ? scores + off : nullptr, ks,
                          keep ? keep + off : nullptr, kk, hist_out ? hist_out + static_cast<size_t>(off) * B : nullptr,
-                         kh, st, cap == 1);
+                         kh, hist_here, st, cap == 1);
       if (rc != COFIE_OK) return rc;
     }
   } else {
@@ -617,7 +628,7 @@ int push_impl(cofie_ngff* h, uint32_t stream, const uint8_t* frames, uint32_t n,
       if (e == cudaSuccess) e = cudaStreamWaitEvent(st, h->ev_copied[slot], 0);
       if (e != cudaSuccess) return h->cuda_fail(e, "host frame staging");
       rc = run_piece(h, stream, h->d_stage[slot], m, scores ? scores + off : nullptr, ks, keep ? keep + off : nullptr,
-                     kk, hist_out ? hist_out + static_cast<size_t>(off) * B : nullptr, kh, st, false);
+                     kk, hist_out ? hist_out + static_cast<size_t>(off) * B : nullptr, kh, hist_here, st, false);
       // the slot is free again only behind whatever of this piece was enqueued, failed or not
       e = cudaEventRecord(h->ev_free[slot], st);
       if (rc != COFIE_OK) return rc;
@@ -960,7 +971,8 @@ int cofie_ngff_push_batch(cofie_ngff_t* h, const cofie_ngff_push_desc* desc, uin
   }
   segs.rows = static_cast<uint32_t>(rows);
   h->shard.ready = false;
-  int rc = run_segments(h, segs, st, false, cap == 1);
+  bool keep_hist = false;
+  int rc = run_segments(h, segs, st, &keep_hist, nullptr, cap == 1);
   if (rc != COFIE_OK) {
     if (host_frames) cudaEventRecord(h->ev_free[slot], st);  // behind whatever of the call was enqueued
     return rc;

@@ -211,6 +211,11 @@ __global__ void __launch_bounds__(kChainThreads) select_chain_kernel(SegTable se
       if (lane == 0) mask[j * W + w] = m;
     }
   }
+  if (a.hist_out) {  // before the map is published: later tiles clear this one's rows after that
+    const uint64_t first_word = static_cast<uint64_t>(j0) * B;
+    for (uint32_t i = tid; i < fn * B; i += kChainThreads)
+      a.hist_out[first_word + i] = kStaged ? rows[L * B + i] : hist_s[first_word + i];
+  }
   __syncthreads();
 
   // 2. the tile's gap map (entry and exit gaps less one, in bytes)

@@ -167,6 +167,7 @@ struct SelectArgs {
   float tau;
   float two_n;        // fp32 of the distance's denominator: 2 W H (histogram), 255 W H (low-res), 64 (dHash)
   uint32_t zero_hist;  // the scan zeroes the push's histogram rows after use
+  uint32_t* hist_out;  // one-stream pushes: the rows are also written here (device; nullptr: not by the selection)
   uint32_t dist_kind;  // 0: sum of |differences| (histogram, low-res); 1: Hamming (dHash)
   uint32_t scd;        // twin-comparison scene changes are added to the rule
   float scd_cut, scd_grad;

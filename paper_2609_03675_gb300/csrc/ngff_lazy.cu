@@ -261,6 +261,11 @@ __global__ void __launch_bounds__(kLazyThreads) lazy_walk_kernel(SegTable segs, 
     ring_s[b] = rows[(n - 1) * P + b];
     if (last) ring_s[B + b] = rows[(last - 1) * P + b];
   }
+  if (a.hist_out)
+    for (uint32_t i = tid; i < n * B; i += kLazyThreads) {
+      const uint32_t r = i / B;
+      a.hist_out[i] = rows[r * P + i - r * B];
+    }
   if (a.zero_hist)
     for (uint32_t i = tid; i < n * B; i += kLazyThreads) feat_s[i] = 0;
 }

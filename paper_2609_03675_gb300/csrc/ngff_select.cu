@@ -556,6 +556,8 @@ __global__ void __launch_bounds__(kWalkThreads) select_walk_kernel(SegTable segs
     state[stream].g = s_g;
     state[stream].acc = s_acc;
   }
+  if (a.hist_out)
+    for (uint32_t i = tid; i < n * B; i += kWalkThreads) a.hist_out[i] = srows[L * B + i];
   if (a.zero_hist) {
     for (uint32_t i = tid; i < n * B; i += kWalkThreads) hist[static_cast<uint64_t>(row0) * B + i] = 0;
   }
