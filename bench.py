@@ -1,5 +1,5 @@
 """NGFF throughput on GB300: frames/s and pixel GB/s of the whole filtering
-path (histogram kernel + windowed-distance kernel + scan kernel) over the
+path (histogram kernel + selection kernel) over the
 1080p stream (3600 uint8 RGB frames of 1920x1080, one whole-stream push).
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl reference]
@@ -612,9 +612,8 @@ def bench_gb300(args):
             "frac_of_nominal_8tbs": pixel_gbs / NOMINAL_HBM_GBS,
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                          "peak_kind": f"{peak_kind} copy bandwidth", "traffic": traffic,
-                         "kernel": ("ngff histogram (K1)" if (spec.width * spec.height) % 16 == 0
-                                    else "ngff histogram, generic kernel (pixel count not a multiple of 16)")
-                         if signal == 0 else f"ngff {args.signal} cell sums (K1 cells)",
+                         "kernel": "ngff histogram (hist_generic_kernel)" if signal == 0
+                         else f"ngff {args.signal} cell sums (K1 cells)",
                          "launch_ms": k1_ms, "bytes_per_launch": k1_bytes,
                          "select_ms_per_step": prof["select_ms"] / max(prof["select_timed"], 1)},
             "e2e": e2e,

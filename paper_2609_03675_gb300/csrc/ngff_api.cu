@@ -1,8 +1,9 @@
 // C ABI of the NGFF library (declared in include/cofie_ngff.h).
 //
 // A push of n frames of one stream runs, in stream order:
-//   memset(hist) -> K1 histograms -> K2 windowed distances + gap masks ->
-//   K3 scan (scores, keep codes, stream state)
+//   the first stage: one feature row per frame (histograms, or a spatial
+//     signal's cells or hash) -> the selection: distances, the rule, scores,
+//     keep codes, stream state, rows cleared for the next push
 // in pieces of at most max_frames_per_push frames. Frames in host memory are
 // copied into one of two device staging buffers on an internal copy stream,
 // overlapping the copy of piece i+1 with the kernels of piece i. Outputs in
@@ -302,8 +303,8 @@ bool first_stage_fast(const cofie_ngff* h, const SegTable& segs) {
   return fast;
 }
 
-// The first stage over the rows of segs: grayscale histograms (K1), or the
-// spatial signal's per-frame features. With pdl the bulk-copy kernels are
+// The first stage over the rows of segs: grayscale histograms, or the spatial
+// signal's per-frame features. With pdl the bulk-copy kernels are
 // programmatic dependents of the kernel before them (they wait for it before
 // reading a frame).
 cudaError_t launch_first_stage(cofie_ngff* h, const SegTable& segs, cudaStream_t st, bool pdl = false) {
@@ -348,8 +349,8 @@ cudaError_t launch_first_stage(cofie_ngff* h, const SegTable& segs, cudaStream_t
   // Which kernel, and the generic kernel's slices (16-pixel groups per CTA).
   // Launches of up to kGenericBins bins, and of frames that K1 does not take:
   //  - fewer than five CTAs of kWaveGroups per SM: slices of 256 groups, as a
-  //    programmatic dependent (pushes of 27 frames of 640x360 in 14.5 us on K1
-  //    12.4; one 4K frame 10.8 on K1, 8.7; 60 frames 19.6 with kWaveGroups,
+  //    programmatic dependent (pushes of 27 frames of 640x360 12.9 us on
+  //    K1, 10.9; one 4K frame 10.8 on K1, 8.7; 60 frames 19.6 with kWaveGroups,
   //    18.3); with many bins to clear and fold 512 from 480,000 groups on (40
   //    frames, 128 bins: 21.3 on kWaveGroups, 20.5 with 256, 19.6 with 512);
   //  - up to one resident wave and an eighth of a second: aligned frames of at
@@ -437,12 +438,12 @@ cudaError_t clear_rows(cofie_ngff* h, uint64_t rows, cudaStream_t st) {
   return cudaMemsetAsync(h->d_hist, 0, static_cast<size_t>(rows) * h->fw * 4, st);
 }
 
-// Runs K1-K3 over the rows described by segs (device frames). Histogram rows
-// are zero between calls, so that a push enqueues the same work whatever came
-// before it (which is what lets a push be captured into a CUDA graph and
-// replayed): the fused small-push kernel clears its rows after use, and
-// otherwise one memset after the selection does, or, with keep_hist, the
-// caller after copying them out. Rows that an earlier call left nonzero (a
+// Runs the first stage and the selection over the rows described by segs
+// (device frames). Histogram rows are zero between calls, so that a push
+// enqueues the same work whatever came before it (which is what lets a push be
+// captured into a CUDA graph and replayed): most selection kernels clear their
+// rows after use, otherwise one memset after the selection does, or, with
+// keep_hist, the caller after copying them out. Rows that an earlier call left nonzero (a
 // prepared shard, a push that failed part way) are cleared first.
 // While `capturing`, nothing here runs until the graph is launched, so the
 // host's record of dirty rows is left as it was and no timing events are taken.
@@ -1113,7 +1114,7 @@ int cofie_ngff_shard_prepare(cofie_ngff_t* h, uint32_t stream, const uint8_t* fr
   DeviceGuard guard(h->device);
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   h->shard.ready = false;
-  // K1 over halo + shard frames; the stream's clock starts at t0 for K2
+  // the first stage over halo + shard frames; the stream's clock starts at t0 for K2
   SegTable all;
   memset(&all, 0, sizeof all);
   all.count = 1;

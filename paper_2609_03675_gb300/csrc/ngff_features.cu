@@ -1,4 +1,4 @@
-// Per-frame kernels around K1: the spatial signals where the streaming
+// Kernels around the histograms: the spatial signals where the streaming
 // kernel does not apply, the dHash bits from cell sums, the bounded-wait
 // probe of the failure path, and the bin check over arbitrary pixels. They
 // share K1's grayscale and bin functions (ngff_device.cuh).

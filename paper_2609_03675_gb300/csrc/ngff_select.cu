@@ -24,14 +24,16 @@
 //    last L_max histograms) is updated at the end, and the push's histogram
 //    rows are zeroed for the next push unless the caller asked for them.
 //
-// Small pushes (at most kSmallMax frames per stream) run K2 and K3 as one
-// kernel: the same CTA first computes its stream's distances, then scans.
-// With at most kWalkMaxFrames frames per stream and L_max <= kWalkMaxLmax the
-// push is smaller still and a lighter kernel decides it (select_walk_kernel):
-// one 256-thread CTA per stream stages the stream's ring and the push's rows
-// in shared memory, keeps the distances and keep bits there, and walks the
-// rule in frame order from the stream's gap, which for so few frames is
-// shorter than composing gap maps.
+// K2 and K3 decide shards and pushes with scene changes (whose runs couple all
+// frames of a push); of those, pushes of at most kSmallMax frames per stream run
+// them as one kernel: the same CTA first computes its stream's distances, then
+// scans. Other pushes of many frames take the tiled selection (ngff_chain.cu).
+// With at most kWalkMaxFrames frames per stream, L_max <= kWalkMaxLmax and rows
+// that fit beside the tables a lighter kernel decides any push
+// (select_walk_kernel): one 256-thread CTA per stream stages the stream's ring
+// and the push's rows in shared memory, keeps the distances and keep bits
+// there, and walks the rule in frame order from the stream's gap, which for so
+// few frames is shorter than composing gap maps.
 #include "ngff_common.cuh"
 
 namespace cofie {
