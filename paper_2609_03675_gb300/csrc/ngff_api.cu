@@ -494,7 +494,7 @@ int run_segments(cofie_ngff* h, const SegTable& segs, cudaStream_t st, bool* kee
     if (e != cudaSuccess) return h->cuda_fail(e, "selection kernel launch");
     h->n_select += 1;
   } else if (chain) {  // tiles of frames, each linked to those before it by their gap maps
-    const ChainArgs ca{h->d_chain_maps, h->d_chain_flags + 2, h->d_chain_flags, h->d_err, kTimeoutNs, 0u, 0u};
+    const ChainArgs ca{h->d_chain_maps, h->d_chain_flags + 2, h->d_chain_flags, h->d_err, kTimeoutNs, 0u, 0u, 0u};
     e = launch_select_chain(segs, sa, ca, h->num_sms, h->d_hist, h->d_ring, h->d_state, st, !ev0);
     if (e != cudaSuccess) return h->cuda_fail(e, "selection kernel launch");
     h->n_select += 1;

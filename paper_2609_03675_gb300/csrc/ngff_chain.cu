@@ -6,10 +6,11 @@
 // possible gap, and a run of frames is a map from the gap before it to the gap
 // after it. The push is cut into tiles of `tile` frames of one stream. A CTA
 // takes one tile:
-//   1. the tile's histogram rows and the L_max rows before them (this push's
-//      rows, or the stream's ring) are copied into shared memory (kStaged) and
-//      the windowed distances L1[j][k-1] = sum_b |c_t - c_{t-k}| and keep bits
-//      computed there, a warp per frame, lane = lag;
+//   1. the tile's histogram rows and the rows before them (this push's rows, or
+//      the stream's ring) are copied into shared memory, for `lags` lags at a
+//      time (all L_max unless the rows are too wide), and the windowed
+//      distances L1[j][k-1] = sum_b |c_t - c_{t-k}| and keep bits computed
+//      there, a warp per frame, lane = lag;
 //   2. the tile's gap map is composed for every entry gap at once (thread =
 //      entry gap), noting the gap before each frame, and published;
 //   3. the entry gap follows from the stream's gap and the maps of the tiles
@@ -28,6 +29,11 @@
 // single-CTA scan of the tables that it wrote and a memset of the rows: 4096
 // frames of 224x224 (B = 32, L_max = 30) pushed in 116 instead of 135 us, 480
 // of 1280x720 (B = 256, L_max = 60) in 211 instead of 236 us.
+// With padded rows a warp reads the frame's word once for its 32 lags: 3000
+// frames of 224x224 (B = 128, L_max = 120) 125 -> 106 us, 8 of 448x448 (L_max =
+// 120) 7.8 -> 7.4 us each from a graph. Rows that do not fit at once, staged for
+// some lags at a time: 1500 frames of 224x224, B = L_max = 256, 723 (rows read
+// from L2 by every lane) -> 159 us.
 #include <algorithm>
 
 #include "ngff_common.cuh"
@@ -38,7 +44,7 @@ namespace {
 constexpr int kChainThreads = 256;
 constexpr uint32_t kChainWarps = kChainThreads / 32;
 constexpr uint32_t kLookBack = 128;            // tiles whose maps a tile composes
-constexpr size_t kChainSmemMax = 200 * 1024;   // rows are staged when everything fits
+constexpr size_t kChainSmemMax = 200 * 1024;   // a CTA's tables and staged rows
 constexpr uint32_t kChainMaxTile = 32;
 
 static_assert(kMaxLmax <= kChainThreads, "a thread per entry gap");
@@ -79,40 +85,45 @@ __device__ __forceinline__ uint32_t flag_wait(const uint32_t* p, uint32_t want, 
   }
 }
 
-__device__ __forceinline__ uint32_t absdiff(uint32_t a, uint32_t b) { return a > b ? a - b : b - a; }
-
-// sum_b |x_b - y_b| by one thread; 16-byte words from the rotated word `rot`
-// on (lanes that read rows B words apart then touch distinct banks).
+// sum_b |x_b - y_b| by one thread (16-byte words with kVec4). x is the same row
+// in every lane; staged rows are padded so that lanes reading the same word of
+// consecutive rows y touch distinct banks.
 template <bool kVec4>
-__device__ __forceinline__ uint32_t row_l1(const uint32_t* x, const uint32_t* y, uint32_t B, uint32_t rot, uint32_t kind) {
+__device__ __forceinline__ uint32_t row_l1(const uint32_t* x, const uint32_t* y, uint32_t B, uint32_t kind) {
   uint32_t d = 0;
   if (kVec4) {
     const uint4* x4 = reinterpret_cast<const uint4*>(x);
     const uint4* y4 = reinterpret_cast<const uint4*>(y);
-    uint32_t q = rot;
 #pragma unroll 8
-    for (uint32_t i = 0; i < B / 4; ++i) {
+    for (uint32_t q = 0; q < B / 4; ++q) {
       const uint4 u = x4[q], v = y4[q];
-      d += absdiff(u.x, v.x) + absdiff(u.y, v.y) + absdiff(u.z, v.z) + absdiff(u.w, v.w);
-      if (++q == B / 4) q = 0;
+      d = __usad(u.x, v.x, d);
+      d = __usad(u.y, v.y, d);
+      d = __usad(u.z, v.z, d);
+      d = __usad(u.w, v.w, d);
     }
   } else if (kind == 1) {  // Hamming distance of bit vectors (dHash)
     for (uint32_t b = 0; b < B; ++b) d += __popc(x[b] ^ y[b]);
   } else {
 #pragma unroll 4
-    for (uint32_t b = 0; b < B; ++b) d += absdiff(x[b], y[b]);
+    for (uint32_t b = 0; b < B; ++b) d = __usad(x[b], y[b], d);
   }
   return d;
 }
 
-// Shared memory, in words: [rows][l1][masks][maps of kLookBack tiles][gap
-// before each frame, by entry gap][the warps' composed maps]
+// Words from one staged row to the next.
+__host__ __device__ constexpr uint32_t chain_stride(uint32_t bins, bool vec4) { return vec4 ? bins + 4 : bins | 1; }
+
+// Shared memory, in words: [the rows that `lags` lags need][the tile's rows, which
+// with all lags at once (lags = l_max) are the last of the rows before][l1]
+// [masks][maps of kLookBack tiles][gap before each frame, by entry gap][the
+// warps' composed maps]
 struct ChainLayout {
-  uint32_t rows, l1, mask, maps, gaps, comp, words;
-  __host__ __device__ ChainLayout(uint32_t tile, uint32_t l_max, uint32_t mask_words, uint32_t bins, bool staged) {
+  uint32_t own, l1, mask, maps, gaps, comp, words;
+  __host__ __device__ ChainLayout(uint32_t tile, uint32_t l_max, uint32_t mask_words, uint32_t stride, uint32_t lags) {
     const uint32_t map_words = 8 * mask_words;  // 32 mask_words entries of one byte
-    rows = 0;
-    l1 = rows + (staged ? (l_max + tile) * bins : 0);
+    own = (lags == l_max ? lags : lags + tile) * stride;
+    l1 = own + tile * stride;
     mask = l1 + tile * l_max;
     maps = mask + tile * mask_words;
     gaps = maps + kLookBack * map_words;
@@ -121,7 +132,8 @@ struct ChainLayout {
   }
 };
 
-template <bool kVec4, bool kStaged>
+// kAll: the rows of all lags at once, staged with the tile's in one pass.
+template <bool kVec4, bool kAll>
 __global__ void __launch_bounds__(kChainThreads) select_chain_kernel(SegTable segs, SelectArgs a, ChainArgs c,
                                                                      uint32_t* __restrict__ hist,
                                                                      uint32_t* __restrict__ ring,
@@ -132,8 +144,11 @@ __global__ void __launch_bounds__(kChainThreads) select_chain_kernel(SegTable se
   const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t B = a.bins, L = a.l_max, W = a.mask_words, F = c.tile;
   const uint32_t stride = 32 * W;  // bytes of a map
-  const ChainLayout lay(F, L, W, B, kStaged);
-  uint32_t* rows = csm + lay.rows;
+  const uint32_t P = chain_stride(B, kVec4);
+  const uint32_t K = kAll ? L : c.lags;  // lags staged at a time: L, or a multiple of 32
+  const ChainLayout lay(F, L, W, P, K);
+  uint32_t* before = csm;            // the rows that the lags at hand need
+  uint32_t* own = csm + lay.own;     // row j of the tile
   uint32_t* l1 = csm + lay.l1;
   uint32_t* mask = csm + lay.mask;
   uint8_t* maps = reinterpret_cast<uint8_t*>(csm + lay.maps);
@@ -164,57 +179,59 @@ __global__ void __launch_bounds__(kChainThreads) select_chain_kernel(SegTable se
   const uint32_t t0_slot = static_cast<uint32_t>(t0 % L);  // ring slot of the push's first frame
   uint32_t* hist_s = hist + static_cast<uint64_t>(sg.row0) * B;
   uint32_t* ring_s = ring + static_cast<uint64_t>(sg.stream) * L * B;
-  // row i of the staged rows is the push's frame j0 - L + i; frames before the
-  // push lie in the ring (slots of frames that never were are read, not used)
+  // the push's frame jj; frames before the push lie in the ring (slots of
+  // frames that never were are read, not used)
   const auto row_of = [&](int32_t jj) -> const uint32_t* {
     if (jj >= 0) return hist_s + static_cast<uint64_t>(jj) * B;
     uint32_t slot = t0_slot + static_cast<uint32_t>(jj + static_cast<int32_t>(L));  // jj >= -L
     if (slot >= L) slot -= L;
     return ring_s + static_cast<uint64_t>(slot) * B;
   };
+  // frames first, first + 1, ... into consecutive staged rows; those more than
+  // L before the push are no frame's lag and left out
+  const auto stage = [&](uint32_t* to, int32_t first, uint32_t rows) {
+    const uint32_t per = kVec4 ? B / 4 : B;
+#pragma unroll 4
+    for (uint32_t i = tid; i < rows * per; i += kChainThreads) {
+      const uint32_t r = i / per, q = i - r * per;
+      const int32_t jj = first + static_cast<int32_t>(r);
+      if (!kAll && jj < -static_cast<int32_t>(L)) continue;
+      if (kVec4)
+        reinterpret_cast<uint4*>(to + r * P)[q] = reinterpret_cast<const uint4*>(row_of(jj))[q];
+      else
+        to[r * P + q] = row_of(jj)[q];
+    }
+  };
 
   // 1. rows, distances, keep bits
-  if (kStaged) {
-    if (kVec4) {
-      const uint32_t nq = B / 4;
-#pragma unroll 4
-      for (uint32_t i = tid; i < (L + fn) * nq; i += kChainThreads) {
-        const uint32_t r = i / nq;
-        reinterpret_cast<uint4*>(rows)[i] =
-            reinterpret_cast<const uint4*>(row_of(static_cast<int32_t>(j0 + r) - static_cast<int32_t>(L)))[i - r * nq];
-      }
-    } else {
-      for (uint32_t i = tid; i < (L + fn) * B; i += kChainThreads) {
-        const uint32_t r = i / B;
-        rows[i] = row_of(static_cast<int32_t>(j0 + r) - static_cast<int32_t>(L))[i - r * B];
-      }
-    }
+  if (!kAll) stage(own, static_cast<int32_t>(j0), fn);
+  for (uint32_t k0 = 0; k0 < (kAll ? 1u : L); k0 += K) {  // lags k0 + 1 .. k0 + K
+    if (!kAll && k0 > 0) __syncthreads();   // the rows of the lags before have been read
+    stage(before, static_cast<int32_t>(j0) - static_cast<int32_t>(k0 + K), kAll ? L + fn : K + fn - 1);
     __syncthreads();
-  }
-  const uint32_t rot = kStaged && kVec4 ? lane % max(B / 4, 1u) : 0u;
-  for (uint32_t j = warp; j < fn; j += kChainWarps) {
-    const unsigned long long t = t0 + j0 + j;
-    const uint32_t* ct = kStaged ? rows + (L + j) * B : row_of(static_cast<int32_t>(j0 + j));
-    uint32_t l_adj = 0;
-    for (uint32_t w = 0; w < W; ++w) {
-      const uint32_t k = 32 * w + lane + 1;
-      const bool valid = k <= L && k <= t;
-      const uint32_t* src = ct;
-      if (valid) src = kStaged ? ct - k * B : row_of(static_cast<int32_t>(j0 + j) - static_cast<int32_t>(k));
-      uint32_t d = row_l1<kVec4>(ct, src, B, rot, a.dist_kind);
-      if (!valid) d = 0;
-      if (w == 0) l_adj = __shfl_sync(0xffffffffu, d, 0);  // lag 1
-      if (k <= L) l1[j * L + k - 1] = d;
-      // fp32(max) / 2N >= tau exactly when max >= x_tau (the smallest such numerator)
-      const bool keep = k <= L && (max(l_adj, d) >= a.x_tau || k >= L);
-      const uint32_t m = __ballot_sync(0xffffffffu, keep);
-      if (lane == 0) mask[j * W + w] = m;
+    for (uint32_t j = warp; j < fn; j += kChainWarps) {
+      const unsigned long long t = t0 + j0 + j;
+      const uint32_t* ct = own + j * P;
+      uint32_t l_adj = !kAll && k0 > 0 ? l1[j * L] : 0u;  // lag 1
+      for (uint32_t w = kAll ? 0 : k0 / 32; kAll ? w < W : 32 * w < min(k0 + K, L); ++w) {
+        const uint32_t k = 32 * w + lane + 1;
+        const bool valid = k <= L && k <= t;
+        uint32_t d = row_l1<kVec4>(ct, valid ? (kAll ? ct - k * P : before + (j + K - (k - k0)) * P) : ct, B, a.dist_kind);
+        if (!valid) d = 0;
+        if (w == 0) l_adj = __shfl_sync(0xffffffffu, d, 0);
+        if (k <= L) l1[j * L + k - 1] = d;
+        // fp32(max) / 2N >= tau exactly when max >= x_tau (the smallest such numerator)
+        const bool keep = k <= L && (max(l_adj, d) >= a.x_tau || k >= L);
+        const uint32_t m = __ballot_sync(0xffffffffu, keep);
+        if (lane == 0) mask[j * W + w] = m;
+      }
     }
   }
   if (a.hist_out) {  // before the map is published: later tiles clear this one's rows after that
-    const uint64_t first_word = static_cast<uint64_t>(j0) * B;
-    for (uint32_t i = tid; i < fn * B; i += kChainThreads)
-      a.hist_out[first_word + i] = kStaged ? rows[L * B + i] : hist_s[first_word + i];
+    for (uint32_t i = tid; i < fn * B; i += kChainThreads) {
+      const uint32_t r = i / B;
+      a.hist_out[static_cast<uint64_t>(j0) * B + i] = own[r * P + i - r * B];
+    }
   }
   __syncthreads();
 
@@ -311,7 +328,7 @@ __global__ void __launch_bounds__(kChainThreads) select_chain_kernel(SegTable se
     const uint32_t keep_n = min(n, L);
     for (uint32_t i = tid; i < keep_n * B; i += kChainThreads) {
       const uint32_t r = i / B, b = i - r * B, jj = n - keep_n + r;
-      const uint32_t v = kStaged ? rows[(L + jj - j0) * B + b] : hist_s[static_cast<uint64_t>(jj) * B + b];
+      const uint32_t v = kAll ? before[(L + jj - j0) * P + b] : hist_s[static_cast<uint64_t>(jj) * B + b];
       ring_s[static_cast<uint64_t>((t0_slot + jj) % L) * B + b] = v;
     }
     __syncthreads();  // the rows below have been copied
@@ -357,12 +374,20 @@ cudaError_t launch_select_chain(const SegTable& segs, const SelectArgs& a, Chain
   c.tile = chain_tile(segs, num_sms);
   c.n_tiles = 0;
   for (uint32_t i = 0; i < segs.count; ++i) c.n_tiles += (segs.s[i].n + c.tile - 1) / c.tile;
-  const bool staged = ChainLayout(c.tile, a.l_max, a.mask_words, a.bins, true).words * sizeof(uint32_t) <= kChainSmemMax;
-  const size_t smem = ChainLayout(c.tile, a.l_max, a.mask_words, a.bins, staged).words * sizeof(uint32_t);
   const bool vec = a.bins % 4 == 0 && a.dist_kind == 0;
-  const auto kernel = vec ? (staged ? select_chain_kernel<true, true> : select_chain_kernel<true, false>)
-                          : (staged ? select_chain_kernel<false, true> : select_chain_kernel<false, false>);
-  const cudaError_t e = launch_dependent(pdl, kernel, dim3(c.n_tiles), dim3(kChainThreads), smem, st, segs, a, c, hist,
+  const uint32_t stride = chain_stride(a.bins, vec);
+  const auto smem = [&](uint32_t lags) {
+    return ChainLayout(c.tile, a.l_max, a.mask_words, stride, lags).words * sizeof(uint32_t);
+  };
+  c.lags = a.l_max;  // every row that a tile reads at once, or as many multiples of 32 lags as fit
+  if (smem(c.lags) > kChainSmemMax) {
+    c.lags = (a.l_max - 1) / 32 * 32;  // below l_max
+    while (c.lags > 32 && smem(c.lags) > kChainSmemMax) c.lags -= 32;
+  }
+  const bool all = c.lags == a.l_max;
+  const auto kernel = vec ? (all ? select_chain_kernel<true, true> : select_chain_kernel<true, false>)
+                          : (all ? select_chain_kernel<false, true> : select_chain_kernel<false, false>);
+  const cudaError_t e = launch_dependent(pdl, kernel, dim3(c.n_tiles), dim3(kChainThreads), smem(c.lags), st, segs, a, c, hist,
                                          ring, state);
   return e == cudaSuccess ? cudaGetLastError() : e;
 }

@@ -189,6 +189,7 @@ struct ChainArgs {
   uint32_t* err;
   uint64_t timeout_ns;
   uint32_t tile, n_tiles;  // frames per tile, tiles of the launch (set by it)
+  uint32_t lags;           // lags whose rows a tile stages at a time (set by the launch)
 };
 
 // Scratch of the selection of larger pushes without forced retention: per row

@@ -1,6 +1,6 @@
 """The selection of larger pushes: tiles of frames linked by their gap maps.
 Pushes around the tile sizes and around the number of tiles that a tile looks
-back on, rows staged in shared memory and not, one and several mask words,
+back on, the rows of all lags staged at once and of some at a time, one and several mask words,
 ring and state carried from push to push, and batches of unequal lengths,
 against the oracle's single pass."""
 import numpy as np
@@ -31,7 +31,8 @@ PUSHES = [[65], [66, 72, 1], [1033, 1024], [1216, 1217], [2432, 70], [2433, 5000
 
 
 @pytest.mark.parametrize("bins,l_max,tau", [(32, 30, 0.15), (32, 1, 0.30), (7, 33, 0.20), (256, 60, 0.50), (32, 256, 0.35),
-                                            (256, 256, 0.60), (4, 64, 2.0), (32, 30, 0.0)])
+                                            (256, 256, 0.60), (256, 161, 0.50), (255, 250, 0.55),
+                                            (4, 64, 2.0), (32, 30, 0.0)])
 @pytest.mark.parametrize("sizes", PUSHES)
 def test_pushes_match_the_oracle(sizes, bins, l_max, tau):
     from paper_2609_03675_gb300 import NGFF
