@@ -175,7 +175,10 @@ __global__ void __launch_bounds__(kChainThreads) select_chain_kernel(SegTable se
   if (!COFIE_BOUND(j0 < n && base + k_tile < c.n_tiles)) return;
   const uint32_t fn = min(F, n - j0);
   const bool last_tile = k_tile + 1 == n_tiles;
+  // the stream's state, read before this tile's map is published: the last tile
+  // writes it once it has seen every map
   const unsigned long long t0 = state[sg.stream].t;
+  const uint32_t g0 = state[sg.stream].g;
   const uint32_t t0_slot = static_cast<uint32_t>(t0 % L);  // ring slot of the push's first frame
   uint32_t* hist_s = hist + static_cast<uint64_t>(sg.row0) * B;
   uint32_t* ring_s = ring + static_cast<uint64_t>(sg.stream) * L * B;
@@ -279,7 +282,7 @@ __global__ void __launch_bounds__(kChainThreads) select_chain_kernel(SegTable se
     __syncthreads();
   }
   if (tid == 0) {
-    uint32_t g = lo > 0 ? s_flag0 >> 2 : state[sg.stream].g;
+    uint32_t g = lo > 0 ? s_flag0 >> 2 : g0;
     if (t0 == 0 && lo == 0) g = 1;
     if (g < 1 || g > L) g = L;  // the state only ever holds [1, L]
     --g;
@@ -340,7 +343,11 @@ __global__ void __launch_bounds__(kChainThreads) select_chain_kernel(SegTable se
     for (uint64_t i = static_cast<uint64_t>(z0) * B + tid; i < static_cast<uint64_t>(z1) * B; i += kChainThreads) hist_s[i] = 0;
   }
   __syncthreads();
-  if (tid == 0) s_bad = atomicAdd(&c.sync[1], 1u) == c.n_tiles - 1;
+  if (tid == 0) {
+    __threadfence();  // this CTA's flags are written before it counts as finished
+    s_bad = atomicAdd(&c.sync[1], 1u) == c.n_tiles - 1;
+    __threadfence();
+  }
   __syncthreads();
   if (s_bad) {  // the last CTA: nobody waits any more
     for (uint32_t i = tid; i < c.n_tiles; i += kChainThreads) c.flags[i] = 0;
