@@ -937,6 +937,21 @@ size_t qer_smem_bytes(uint32_t n_pad) {
   return static_cast<size_t>(qer_stages(n_pad)) * qer_stage_bytes(n_pad) + 1024;  // + slack for 1024-B alignment
 }
 
+// The limits that a kernel's launches may ask for belong to the kernel, not to
+// a handle: every handle sets the same ones, the largest of any text block and
+// dot product length, so that creating one never lowers another's. Launches
+// and residency go by each handle's own sizes, which stay within these.
+constexpr size_t kQerSmemLimit = kQerStageBudget + 1024;
+constexpr size_t kQerPairSmemLimit = kQerPairRingBudget + 1024;
+
+cudaError_t qer_smem_limits() {
+  cudaError_t e = cudaFuncSetAttribute(qer_score, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kQerSmemLimit));
+  for (const auto k : {qer_score_pair<1>, qer_score_pair<2>})
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kQerPairSmemLimit));
+  return e;
+}
+
 PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
   static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
   if (!fn) {
@@ -1119,8 +1134,8 @@ int cofie_qer_create(const cofie_qer_params* p, cofie_qer_t** out) {
   if (e == cudaSuccess) e = cudaMemset(h->d_done, 0, sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMalloc(&h->d_err, sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMemset(h->d_err, 0, sizeof(uint32_t));
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(qer_score, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(h->smem));
+  if (e == cudaSuccess) e = qer_smem_limits();
+  if (e == cudaSuccess && h->smem > kQerSmemLimit) e = cudaErrorInvalidConfiguration;
   int per_sm_ctas = 0, n_sms = 0;
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_ctas, qer_score, kQerThreads, h->smem);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, dev);
@@ -1140,8 +1155,7 @@ int cofie_qer_create(const cofie_qer_params* p, cofie_qer_t** out) {
     const int pair_ctas_by_tmem = static_cast<int>(512 / (2 * h->acc_cols));
     while (per_sm / (h->pair_smem + 1024) > static_cast<size_t>(pair_ctas_by_tmem)) h->pair_smem += 1024;
     const auto pair_fn = h->pair_sub == 2 ? qer_score_pair<2> : qer_score_pair<1>;  // the one launched
-    cudaError_t pe = cudaFuncSetAttribute(pair_fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          static_cast<int>(h->pair_smem));
+    cudaError_t pe = h->pair_smem > kQerPairSmemLimit ? cudaErrorInvalidConfiguration : cudaSuccess;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 2;

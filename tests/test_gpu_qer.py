@@ -314,3 +314,27 @@ def test_selection_by_rank(n, values):
         order = real[np.lexsort((real, -w[real]))][:kk]
         assert np.array_equal(sel.cpu().numpy(), np.sort(np.concatenate([order, np.flatnonzero(np.isnan(w))])))
         g.close()
+
+
+@pytest.mark.parametrize("texts", [(256, 64, 40, 16), (16, 40, 64, 256)])
+@pytest.mark.parametrize("d", [64, 128])
+def test_handles_of_different_text_lengths_alive_together(texts, d):
+    """The scoring kernels ask for shared memory by the text block and the dot
+    product length. With handles of several text lengths alive, made in
+    falling and rising order, each runs at frame counts on the paired kernel
+    and on the one-SM kernel after all of them exist, with the result that it
+    gives alone."""
+    from paper_2609_03675_gb300 import QER
+    runs = []
+    for n_text in texts:
+        spec = S.QerSpec(n_text=n_text, n_heads=d // 16, n_kv_heads=d // 64, head_dim=64, n_frames=120, tokens_per_frame=256,
+                         seed=n_text)
+        q, k, _ = S.generate(spec)
+        q, k = torch.from_numpy(q.view(np.int16)).cuda(), torch.from_numpy(k.view(np.int16)).cuda()
+        f = QER(n_text, spec.n_heads, spec.n_kv_heads, 64, 120, 256, 0.3)
+        runs.append((f, q, k, [[x.clone() for x in f.run(q, k[: n * 256])] for n in (20, 120)]))
+    for f, q, k, alone in runs:
+        for n, (w0, s0) in zip((20, 120), alone):
+            w, s = f.run(q, k[: n * 256])
+            assert torch.equal(w, w0) and torch.equal(s, s0)
+        f.status()
