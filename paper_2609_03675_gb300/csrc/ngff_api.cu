@@ -836,7 +836,7 @@ int cofie_ngff_create(const cofie_ngff_params* p, cofie_ngff_t** out) {
   if (e == cudaSuccess && chained) e = cudaMemset(h->d_chain_flags, 0, chain_flags * sizeof(uint32_t));
   if (e == cudaSuccess && chained) e = chain_prepare();
   if (e == cudaSuccess && p->l_max == 0) e = lazy_prepare();
-  if (e == cudaSuccess && p->l_max > 0) e = scan_prepare(h->mask_words, p->l_max);
+  if (e == cudaSuccess && p->l_max > 0) e = scan_prepare();
   if (e == cudaSuccess && h->bin_path >= 0) {
     const int per_sm = hist_blocks_per_sm(h->bin_path, p->bins);
     if (per_sm <= 0) e = cudaGetLastError() != cudaSuccess ? cudaErrorInvalidConfiguration : cudaErrorInvalidValue;

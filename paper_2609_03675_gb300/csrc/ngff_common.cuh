@@ -298,7 +298,7 @@ cudaError_t launch_lazy_select(const SegTable& segs, const SelectArgs& a, uint32
                                const uint32_t* feat, uint32_t* ring, StreamState* state, cudaStream_t st, bool pdl = false);
 cudaError_t launch_debug_bins(const uint8_t* px, uint64_t n_groups, const LumaConsts& lc, int bin_path,
                               uint8_t* bins_out, cudaStream_t st);
-cudaError_t scan_prepare(uint32_t mask_words, uint32_t l_max);
+cudaError_t scan_prepare();
 cudaError_t launch_gap_map(const Segment& seg, const SelectArgs& a, unsigned long long t0, const uint32_t* mask,
                            uint16_t* map_out, cudaStream_t st);
 cudaError_t launch_ring_store(const uint32_t* hist, uint32_t rows, unsigned long long t_first, uint32_t stream,

@@ -658,15 +658,9 @@ cudaError_t launch_select_walk(const SegTable& segs, const SelectArgs& a, uint32
 cudaError_t launch_gap_map(const Segment& seg, const SelectArgs& a, unsigned long long t0, const uint32_t* mask,
                            uint16_t* map_out, cudaStream_t st) {
   const size_t smem = scan_smem_bytes(a.mask_words, a.l_max);
-  cudaError_t e;
-  if (a.mask_words == 1) {
-    e = cudaFuncSetAttribute(gap_map_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-    if (e == cudaSuccess) gap_map_kernel<true><<<1, kScanThreads, smem, st>>>(seg, a, t0, mask, map_out);
-  } else {
-    e = cudaFuncSetAttribute(gap_map_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-    if (e == cudaSuccess) gap_map_kernel<false><<<1, kScanThreads, smem, st>>>(seg, a, t0, mask, map_out);
-  }
-  return e == cudaSuccess ? cudaGetLastError() : e;
+  const auto kernel = a.mask_words == 1 ? gap_map_kernel<true> : gap_map_kernel<false>;
+  kernel<<<1, kScanThreads, smem, st>>>(seg, a, t0, mask, map_out);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_ring_store(const uint32_t* hist, uint32_t rows, unsigned long long t_first, uint32_t stream,
@@ -676,25 +670,21 @@ cudaError_t launch_ring_store(const uint32_t* hist, uint32_t rows, unsigned long
   return cudaGetLastError();
 }
 
-cudaError_t scan_prepare(uint32_t mask_words, uint32_t l_max) {
-  const int smem = static_cast<int>(scan_smem_bytes(mask_words, l_max));
-  cudaError_t e = cudaFuncSetAttribute(select_walk_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWalkSmemMax);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(select_walk_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWalkSmemMax);
-  if (e != cudaSuccess) return e;
-  if (mask_words == 1) {
-    e = cudaFuncSetAttribute(scan_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(select_small_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(select_small_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  } else {
-    e = cudaFuncSetAttribute(scan_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(select_small_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(select_small_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  }
+// The limits belong to the kernels, not to a handle: every handle sets the same
+// ones, the largest that any L_max takes. With one mask word (26 KiB) the
+// default of 48 KiB does.
+cudaError_t scan_prepare() {
+  cudaError_t e = cudaSuccess;
+  const auto limit = [&](const auto k, size_t bytes) {
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+  };
+  const size_t scan = scan_smem_bytes(kMaxLmax / 32, kMaxLmax);
+  limit(select_walk_kernel<true>, kWalkSmemMax);
+  limit(select_walk_kernel<false>, kWalkSmemMax);
+  limit(scan_kernel<false>, scan);
+  limit(select_small_kernel<true, false>, scan);
+  limit(select_small_kernel<false, false>, scan);
+  limit(gap_map_kernel<false>, scan);
   return e;
 }
 

@@ -189,3 +189,29 @@ def test_gradual_threshold_at_or_above_the_cut(t_cut, t_grad, l_max):
                  max_frames_per_push=T)
         sg, kg = _run(f, dev, chunks)
         _assert_same(sg, kg, so, ko, f"T_b {t_cut} T_s {t_grad} L_max {l_max} {chunks[:2]}")
+
+
+@pytest.mark.parametrize("order", [(120, 45, 30, 7), (7, 30, 45, 120)])
+def test_handles_of_different_gap_limits_alive_together(order):
+    """The scan kernels and the gap-map kernel ask for shared memory by L_max.
+    With handles of several limits alive, each decides pushes of 40 frames
+    (fused beyond L_max = 64) and 100 frames (window + scan) after all of them
+    exist, and shards are prepared and committed on plain handles made in
+    the same order."""
+    from paper_2609_03675_gb300 import NGFF, _abi
+    T = 140
+    fr = _frames_from_positions(_walk(T, seed=77))
+    dev = torch.from_numpy(fr).cuda()
+    scenes = {L: NGFF(W, H, tau=0.5, l_max=L, signal=_abi.SIGNAL_SCD, scd_cut=0.125, scd_gradual=0.01) for L in order}
+    plain = {L: NGFF(W, H, tau=0.1, l_max=L) for L in order}
+    for L, f in scenes.items():
+        so, ko = _oracle(fr, O.Params(W, H, tau=0.5, l_max=L), 0.125, 0.01)
+        sg, kg = _run(f, dev, [40, 100])
+        _assert_same(sg, kg, so, ko, f"L_max {L}")
+    for L, f in plain.items():
+        _, so, ko = O.load().run(fr, O.Params(W, H, tau=0.1, l_max=L))
+        f.shard_prepare(dev, n_halo=0, t0=0)
+        s, k = f.shard_commit(1, T)
+        torch.cuda.synchronize()
+        f.status()
+        _assert_same(s.cpu().numpy().astype(np.float64), k.cpu().numpy(), so, ko, f"shard, L_max {L}")
