@@ -17,8 +17,9 @@
 //     stream's reference: within blocks of 32 frames by pointer doubling for
 //     all entries at once, then one step per block. A link that the staged
 //     rows did not settle (no keep for many frames) is scanned for by the
-//     whole CTA. Scene changes depend only on the adjacent distances and are
-//     found first, by a scan of the twin comparison's run;
+//     whole CTA, as far as the next scene change. Scene changes depend only on
+//     the adjacent distances and are found first, by a scan of the twin
+//     comparison's run;
 //   lazy_emit_kernel   with every frame's reference known, scores and keep
 //     codes, eight lanes per frame.
 // Bound by latency, as the other selections are. A walk by one warp, a window
@@ -48,6 +49,8 @@ constexpr uint32_t kLinkWarps = kLinkThreads / 32;
 constexpr uint32_t kLinkBlocks = 128;              // blocks of 32 frames per pass of the chain kernel
 constexpr uint32_t kLinkTile = 32 * kLinkBlocks;
 constexpr uint32_t kPer = kLinkBlocks / kLinkWarps;  // blocks per warp
+constexpr uint32_t kScanFrames = kLinkThreads / 8;   // frames per pass of an open link's scan, four times as many
+constexpr uint32_t kScanNarrow = 64;                 // with rows of at most 64 words
 constexpr uint32_t kUnknown = 0xffffffffu;         // no keep among the staged rows, but frames beyond them
 
 __device__ __forceinline__ uint32_t word_dist(uint32_t x, uint32_t y, uint32_t kind) {
@@ -350,6 +353,58 @@ __global__ void __launch_bounds__(kLazyThreads) lazy_next_kernel(SegTable segs, 
   }
 }
 
+// kN * kScanFrames frames from f0 on, eight lanes per frame: those before
+// `stop` whose distances reach the threshold lower *found. True in the lanes
+// that found one. Bound by the latency of a pass, so passes are short (a keep
+// is near more often than not) and rows are read in whole lines: stills of 64x64
+// with 256 bins and scenes 80 frames apart, whose links all have to be scanned
+// for, take 191 us for 4096 frames and 643 us for 16384 (walked by one warp 580
+// and 2247 us; with a thread per row and every scan on to the push's end, past
+// the scene changes, 3.6 and 86 ms).
+template <bool kVec4, uint32_t kN>
+__device__ __forceinline__ bool scan_pass(const uint32_t* feat_s, const uint32_t* adj, const uint32_t* ref, uint32_t f0,
+                                          uint32_t stop, const SelectArgs& a, uint32_t* found) {
+  const uint32_t sub = threadIdx.x & 7, B = a.bins;
+  const uint32_t* row[kN];
+  uint32_t d[kN], d_adj[kN];
+#pragma unroll
+  for (uint32_t u = 0; u < kN; ++u) {
+    const uint32_t f = min(f0 + u * kScanFrames + (threadIdx.x >> 3), stop - 1);
+    row[u] = feat_s + static_cast<uint64_t>(f) * B;
+    d_adj[u] = adj[f];
+    d[u] = 0;
+  }
+  if (kVec4) {
+#pragma unroll(kN == 1 ? 8 : 1)
+    for (uint32_t q = sub; q < B / 4; q += 8) {
+      const uint4 v = reinterpret_cast<const uint4*>(ref)[q];
+#pragma unroll
+      for (uint32_t i = 0; i < kN; ++i) {
+        const uint4 u = reinterpret_cast<const uint4*>(row[i])[q];
+        d[i] += word_dist(u.x, v.x, 0) + word_dist(u.y, v.y, 0) + word_dist(u.z, v.z, 0) + word_dist(u.w, v.w, 0);
+      }
+    }
+  } else {
+#pragma unroll 4
+    for (uint32_t b = sub; b < B; b += 8) {
+#pragma unroll
+      for (uint32_t i = 0; i < kN; ++i) d[i] += word_dist(row[i][b], ref[b], a.dist_kind);
+    }
+  }
+  bool any = false;
+#pragma unroll
+  for (uint32_t u = 0; u < kN; ++u) {
+#pragma unroll
+    for (uint32_t o = 4; o > 0; o >>= 1) d[u] += __shfl_xor_sync(0xffffffffu, d[u], o);
+    const uint32_t f = f0 + u * kScanFrames + (threadIdx.x >> 3);
+    if (f < stop && max(d_adj[u], d[u]) >= a.x_tau) {
+      any = true;
+      if (sub == 0) atomicMin(found, f);
+    }
+  }
+  return any;
+}
+
 template <bool kVec4>
 __global__ void __launch_bounds__(kLinkThreads) lazy_chain_kernel(SegTable segs, SelectArgs a, LazyArgs z,
                                                                   const uint32_t* __restrict__ feat,
@@ -365,7 +420,7 @@ __global__ void __launch_bounds__(kLinkThreads) lazy_chain_kernel(SegTable segs,
   __shared__ uint32_t breset[kLinkBlocks];
   __shared__ unsigned long long bsum[kLinkBlocks];
   __shared__ unsigned long long s_acc;
-  __shared__ uint32_t s_at, s_ref, s_found, s_last;
+  __shared__ uint32_t s_at, s_last, s_start, s_stop, s_found;
   pdl_trigger();
   const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const Segment& sg = segs.s[blockIdx.x];
@@ -500,7 +555,9 @@ __global__ void __launch_bounds__(kLinkThreads) lazy_chain_kernel(SegTable segs,
       visit[f] = mask;
     }
     __syncthreads();
-    // one step per block; a link still open is scanned for by the whole CTA
+    // one step per block; a link still open is scanned for by the whole CTA, as
+    // far as the first scene change or the tile's end: a reference without a
+    // keep until there is scanned for on in the next tile
     for (;;) {
       if (tid == 0) {
         uint32_t r = s_at, last = s_last;
@@ -512,40 +569,32 @@ __global__ void __launch_bounds__(kLinkThreads) lazy_chain_kernel(SegTable segs,
         }
         s_at = r;
         s_last = last;
-        s_ref = last;
+        if (r == kUnknown) {  // the reference is frame last - 1 (or the stream's, last = 0)
+          const uint32_t from = last > c0 ? last - c0 : 0;  // local frames from here on
+          uint32_t scene = kUnknown;
+          if (from < m) {
+            const uint32_t blk = from >> 5, up = scenes[blk] & (0xffffffffu << (from & 31));
+            scene = up ? c0 + 32 * blk + __ffs(up) - 1 : after[blk];
+          }
+          // the first frame that was neither staged with it nor scanned in an earlier tile
+          s_start = max(c0, last ? resume(last - 1) : min(n, z.stage_rows - 1));
+          s_found = s_stop = min(scene, c1);
+        }
       }
       __syncthreads();
       if (s_at != kUnknown) break;
-      // the reference is frame s_ref - 1 (or the stream's, s_ref = 0): its
-      // first keep at or past the first frame that was not staged with it
-      const uint32_t ref1 = s_ref;
-      const uint32_t* ref = ref1 ? feat_s + static_cast<uint64_t>(ref1 - 1) * B : old_ref;
-      const uint32_t start = ref1 ? resume(ref1 - 1) : min(n, z.stage_rows - 1);
-      uint32_t found = n;
-      for (uint32_t f0 = start; f0 < n; f0 += kLinkThreads) {
-        __syncthreads();
-        if (tid == 0) s_found = n;
-        __syncthreads();
-        const uint32_t f = f0 + tid;
-        if (f < n && max(z.adj[row0 + f], row_dist<kVec4>(feat_s + static_cast<uint64_t>(f) * B, ref, B, 0u, a.dist_kind)) >= a.x_tau)
-          atomicMin(&s_found, f);
-        __syncthreads();
-        found = s_found;
-        if (found < n) break;
+      const uint32_t stop = s_stop;
+      const uint32_t* ref = s_last ? feat_s + static_cast<uint64_t>(s_last - 1) * B : old_ref;
+      const uint32_t per = B <= kScanNarrow ? 4 * kScanFrames : kScanFrames;
+      for (uint32_t f0 = s_start; f0 < stop; f0 += per) {
+        const bool keep = B <= kScanNarrow ? scan_pass<kVec4, 4>(feat_s, z.adj + row0, ref, f0, stop, a, &s_found)
+                                           : scan_pass<kVec4, 1>(feat_s, z.adj + row0, ref, f0, stop, a, &s_found);
+        if (__syncthreads_or(keep)) break;
       }
+      const uint32_t found = s_found;
       __syncthreads();
-      if (tid == 0) {
-        // a scene change of this tile past the reference comes first; a later
-        // tile's is looked at when that tile is entered
-        uint32_t scene = kUnknown;
-        const uint32_t from = ref1 > c0 ? ref1 - c0 : 0;  // local frames from here on
-        if (from < m) {
-          const uint32_t blk = from >> 5, up = scenes[blk] & (0xffffffffu << (from & 31));
-          scene = up ? c0 + 32 * blk + __ffs(up) - 1 : after[blk];
-        }
-        s_at = min(found, scene);
-      }
-      __syncthreads();
+      if (found == c1 && c1 < n) break;  // open still
+      if (tid == 0) s_at = found;
     }
     __syncthreads();
     if (warp == 0) {  // the last kept frame before each block: a prefix maximum over blocks

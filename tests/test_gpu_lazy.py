@@ -175,3 +175,57 @@ def test_batch_of_unequal_lengths_without_gap():
         _, so, ko = O.load().run(frs[s], O.Params(32, 8, tau=0.06, l_max=0))
         assert np.array_equal(outs[s][1].cpu().numpy(), ko), s
         assert (np.abs(outs[s][0].cpu().numpy().astype(np.float64) - so) <= SCORE_RTOL * so).all(), s
+
+
+@pytest.mark.parametrize("bins,tau,apart", [(256, 3.0, 80), (256, 0.3, 80), (32, 3.0, 700), (32, 0.3, 700), (6, 3.0, 300),
+                                            (256, 3.0, 5000)])
+@pytest.mark.parametrize("chunks", [[9000], [4096, 4904], [300, 4200, 4500]])
+def test_scenes_far_apart(chunks, bins, tau, apart):
+    """Stills whose scenes lie further apart than the rows that are staged with
+    a reference, so that nearly every link is scanned for: up to a scene
+    change (no novelty at tau = 3), to a novelty keep, and on over the chain's
+    passes of 4096 frames and from push to push."""
+    from paper_2609_03675_gb300 import NGFF, _abi
+    w, h, T = 32, 8, sum(chunks)
+    fr = _frames(w, h, T, seed=820 + bins, mean=apart)
+    for a in range(0, T, apart):
+        fr[a:a + apart] = fr[a]
+    fr[5::apart // 3, 0, 0] ^= 1  # a few small differences within the scenes
+    p = O.Params(w, h, bins=bins, tau=tau, l_max=0)
+    hist = np.stack([O.load().histogram(x, p) for x in fr])
+    so, ko = SC.select(hist, p, 0.2, 0.1)
+    assert (ko != 0).sum() > T // apart // 3
+    f = NGFF(w, h, bins=bins, tau=tau, l_max=0, max_frames_per_push=max(chunks), signal=_abi.SIGNAL_SCD, scd_cut=0.2,
+             scd_gradual=0.1)
+    got = [f.push(part) for part in torch.split(torch.from_numpy(fr).cuda(), chunks)]
+    torch.cuda.synchronize()
+    f.status()
+    kg = torch.cat([k for _, k in got]).cpu().numpy()
+    assert np.array_equal(kg, ko), np.flatnonzero(kg != ko)[:10]
+    assert (np.abs(torch.cat([s for s, _ in got]).cpu().numpy().astype(np.float64) - so) <= SCORE_RTOL * so).all()
+
+
+def test_scan_time_grows_with_the_frames():
+    """No frame is scanned for more than one reference: four times the frames
+    with the same distance between scenes take about four times as long, not
+    sixteen (as when every reference's scan ran to the end of the push)."""
+    from paper_2609_03675_gb300 import NGFF, _abi
+    w, h, apart, us = 32, 8, 80, []
+    for T in (4096, 16384):
+        f = NGFF(w, h, bins=256, tau=3.0, l_max=0, max_frames_per_push=T, signal=_abi.SIGNAL_SCD)
+        still = torch.randint(0, 256, (T // apart + 1, h, w, 3), dtype=torch.uint8, device="cuda")
+        fr = still.repeat_interleave(apart, dim=0)[:T].contiguous()
+        out = dict(scores=torch.empty(T, device="cuda"), keep=torch.empty(T, dtype=torch.uint8, device="cuda"))
+        times = []
+        for _ in range(9):
+            f.reset()
+            a, b = torch.cuda.Event(True), torch.cuda.Event(True)
+            a.record()
+            f.push(fr, **out)
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b))
+        f.status()
+        assert int((out["keep"] != 0).sum()) == (T + apart - 1) // apart
+        us.append(sorted(times)[4])
+    assert us[1] < 8 * us[0], us
