@@ -448,8 +448,7 @@ cudaError_t clear_rows(cofie_ngff* h, uint64_t rows, cudaStream_t st) {
 // While `capturing`, nothing here runs until the graph is launched, so the
 // host's record of dirty rows is left as it was and no timing events are taken.
 // keep_hist is cleared when the selection has written the rows to hist_out
-// itself (device memory of the handle's device, a push of one stream) and
-// zeroed them.
+// itself (a push of one stream, see push_impl for the memory) and zeroed them.
 int run_segments(cofie_ngff* h, const SegTable& segs, cudaStream_t st, bool* keep_hist, uint32_t* hist_out, bool capturing) {
   if (segs.rows == 0) return COFIE_OK;
   cudaError_t e = clear_rows(h, h->dirty_rows, st);
@@ -523,7 +522,7 @@ int run_segments(cofie_ngff* h, const SegTable& segs, cudaStream_t st, bool* kee
 }
 
 // One piece of a single-stream push: n <= max_frames_per_push device frames.
-// hist_here: hist_out is memory of the handle's device.
+// hist_here: hist_out is memory that kernels of the handle's device can write.
 int run_piece(cofie_ngff* h, uint32_t stream, const uint8_t* dframes, uint32_t n, float* scores, MemKind ks,
               uint8_t* keep, MemKind kk, uint32_t* hist_out, MemKind kh, bool hist_here, cudaStream_t st, bool capturing) {
   SegTable segs;
@@ -594,8 +593,15 @@ int push_impl(cofie_ngff* h, uint32_t stream, const uint8_t* frames, uint32_t n,
   int fdev = -1;
   const MemKind kf = classify(frames, &fdev);
   int hdev = -1;
-  const MemKind ks = classify(scores), kk = classify(keep), kh = classify(hist_out, &hdev);
-  const bool hist_here = kh == kDevice && hdev == h->device;
+  KindRange hist_in;
+  const MemKind ks = classify(scores), kk = classify(keep), kh = classify_in(hist_out, &hdev, &hist_in);
+  // The selection may write rows to hist_out itself where a kernel's stores are
+  // as good as a copy: words on the handle's device, aligned, inside one
+  // allocation from the first to the last. Everything else is left to the copy,
+  // which takes any alignment and refuses a range past its allocation.
+  const uintptr_t hist_at = reinterpret_cast<uintptr_t>(hist_out);
+  const bool hist_here = kh == kDevice && hdev == h->device && hist_at % 4 == 0 && hist_at >= hist_in.lo &&
+                         hist_at < hist_in.hi && static_cast<uint64_t>(n) * h->fw * 4 <= hist_in.hi - hist_at;
   if (kf == kDevice && fdev != h->device) return h->fail(COFIE_EINVAL, "frames live on another device");
   const int cap = capture_state(st);
   if (cap < 0) return h->fail(COFIE_ECUDA, "cannot read the CUDA stream's capture state");

@@ -271,3 +271,25 @@ def test_histogram_rows_cleared_between_pushes():
     assert np.array_equal(torch.cat(got_k).cpu().numpy(), ko)
     s = torch.cat(got_s).cpu().numpy().astype(np.float64)
     assert np.all(np.abs(s - so) <= 1e-6 * so)
+
+
+@pytest.mark.parametrize("n,l_max", [(20, 30), (100, 30), (20, 0), (300, 0)])
+@pytest.mark.parametrize("shift", [0, 1, 2, 3])
+def test_histograms_into_memory_off_the_word_boundaries(n, l_max, shift):
+    """The C entry point's hist_out at any byte offset, on every selection
+    kernel: on a word boundary the selection writes the rows, off it a copy
+    does. Bytes around the rows stay untouched."""
+    fr = synth.generate(synth.medium(seed=43).with_(width=48, height=32, frames=2 * n, mean_scene_len=12))
+    ho, _, ko = oracle_run(fr, O.Params(48, 32, tau=0.05, l_max=l_max))
+    dev = torch.from_numpy(fr).cuda()
+    keep = torch.empty(2 * n, dtype=torch.uint8, device="cuda")
+    f = _ngff(48, 32, tau=0.05, l_max=l_max)
+    for a in (0, n):
+        out = torch.full((n * 128 + 16,), 7, dtype=torch.uint8, device="cuda")
+        f.push_raw(0, dev[a:a + n].data_ptr(), n, None, keep[a:a + n].data_ptr(), out.data_ptr() + 4 + shift)
+        got = out.cpu().numpy()
+        rows = got[4 + shift:4 + shift + n * 128].copy().view(np.uint32).reshape(n, 32)
+        assert np.array_equal(rows, ho[a:a + n])
+        assert (got[:4 + shift] == 7).all() and (got[4 + shift + n * 128:] == 7).all()
+    f.status()
+    assert np.array_equal(keep.cpu().numpy(), ko)
