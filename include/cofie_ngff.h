@@ -554,6 +554,14 @@ int cofie_qer_profile_reset(cofie_qer_t* h, int time_kernels);
 int cofie_qer_profile_read(cofie_qer_t* h, uint64_t* launches, uint64_t* timed, double* score_ms, double* flops,
                            double* key_bytes);
 
+/*
+ * Test hook for the failure path, as cofie_ngff_debug_fail_alloc: after >= 0:
+ * that many further kernel launches of cofie_qer_run succeed and the next one
+ * is refused on the host (the call returns COFIE_ECUDA and launches nothing
+ * after it). after < 0 switches it off.
+ */
+void cofie_qer_debug_fail_launch(int32_t after);
+
 /* Last error of h, or of the last failed cofie_qer_create when h is NULL. Never NULL. */
 const char* cofie_qer_last_error(const cofie_qer_t* h);
 

@@ -48,6 +48,7 @@ EXPORTS = (
     "cofie_ngff_global_error",
     "cofie_qer_create",
     "cofie_qer_destroy",
+    "cofie_qer_debug_fail_launch",
     "cofie_qer_run",
     "cofie_qer_status",
     "cofie_qer_kernel_in_use",
@@ -193,6 +194,8 @@ def load():
     lib.cofie_qer_create.restype = ctypes.c_int
     lib.cofie_qer_destroy.argtypes = [H]
     lib.cofie_qer_destroy.restype = None
+    lib.cofie_qer_debug_fail_launch.argtypes = [ctypes.c_int32]
+    lib.cofie_qer_debug_fail_launch.restype = None
     lib.cofie_qer_run.argtypes = [H, vp, vp, u32, vp, vp, vp, vp]
     lib.cofie_qer_run.restype = ctypes.c_int
     lib.cofie_qer_status.argtypes = [H, vp]

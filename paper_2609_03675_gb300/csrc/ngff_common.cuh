@@ -237,16 +237,18 @@ struct NvtxRange {
   NvtxRange& operator=(const NvtxRange&) = delete;
 };
 
-// Host-side fault injection for tests: when >= 0, that many further device
-// allocations of the library succeed and the next one fails (then the hook
-// switches itself off). Set through cofie_ngff_debug_fail_alloc.
-extern std::atomic<int> g_fail_alloc;
-inline bool injected_alloc_failure() {
-  int left = g_fail_alloc.load();
-  while (left >= 0 && !g_fail_alloc.compare_exchange_weak(left, left - 1)) {
+// Host-side fault injection for tests: when `hook` is >= 0, that many further
+// operations succeed and the next one fails (then the hook switches itself
+// off).
+inline bool injected_failure(std::atomic<int>& hook) {
+  int left = hook.load();
+  while (left >= 0 && !hook.compare_exchange_weak(left, left - 1)) {
   }
   return left == 0;
 }
+// Device allocations of the library, set through cofie_ngff_debug_fail_alloc.
+extern std::atomic<int> g_fail_alloc;
+inline bool injected_alloc_failure() { return injected_failure(g_fail_alloc); }
 
 // Launchers (stream-ordered; return the launch error).
 int hist_blocks_per_sm(int bin_path, uint32_t bins);  // K1's resident CTAs (-1 on error)

@@ -1068,6 +1068,7 @@ void qer_free(cofie_qer* h) {
 }
 
 thread_local std::string g_qer_error;
+std::atomic<int> g_fail_launch{-1};  // see cofie_qer_debug_fail_launch
 
 }  // namespace
 
@@ -1196,6 +1197,8 @@ int cofie_qer_create(const cofie_qer_params* p, cofie_qer_t** out) {
 
 void cofie_qer_destroy(cofie_qer_t* h) { qer_free(h); }
 
+void cofie_qer_debug_fail_launch(int32_t after) { g_fail_launch.store(after < 0 ? -1 : after); }
+
 uint32_t cofie_qer_kernel_in_use(const cofie_qer_t* h) {
   return h ? (h->pair ? COFIE_QER_KERNEL_PAIR : COFIE_QER_KERNEL_ONE_SM) : 0u;
 }
@@ -1243,14 +1246,41 @@ int cofie_qer_run(cofie_qer_t* h, const uint16_t* q, const uint16_t* k, uint32_t
   const uint32_t q_box = pair_run ? n_pad / 2 : n_pad;  // the pair's CTAs each stage half of q~
   if (!make_map(&map_k, k, nv, h->D, kQerM)) return h->fail(COFIE_ECUDA, "tensor map encoding failed");
   const uint32_t n_rows = h->n_blk * h->n_pad;
+  // Every kernel may be scheduled while its predecessor still runs, and waits
+  // for it (griddepcontrol.wait) where it reads what that kernel or one before
+  // it wrote: every thread of the first kernel, which lets the scoring kernel
+  // start only after its wait, so that the keys are ready when that one does;
+  // the scoring kernel's q~ producer; every thread of the mean and ranking
+  // kernels. With the timing events in between, the scoring kernel's launch
+  // serialises as usual.
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = 2;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cfg.blockDim = dim3(256, 1, 1);
+  // A launch that fails ends the call: the kernels after it would work on what
+  // an earlier call left in the scratch.
+  cudaError_t e = cudaSuccess;
+  const auto launch = [&](auto kernel, auto... args) {
+    if (e == cudaSuccess)
+      e = injected_failure(g_fail_launch) ? cudaErrorLaunchOutOfResources : cudaLaunchKernelEx(&cfg, kernel, args...);
+  };
   if (p.head_dim % 8 == 0 && reinterpret_cast<uintptr_t>(q) % 16 == 0) {
     const uint64_t n8 = static_cast<uint64_t>(n_rows) * h->D / 8;
     const uint32_t blocks = static_cast<uint32_t>(std::min<uint64_t>((n8 + 255) / 256, 1024));
-    launch_dependent(true, qer_prepare_q8, dim3(blocks), dim3(256), 0, st, reinterpret_cast<const uint4*>(q), p.n_text,
-                     n_rows, h->n_pad, h->per_blk, p.n_heads, p.n_kv_heads, p.head_dim, reinterpret_cast<uint4*>(h->d_qg));
+    cfg.gridDim = dim3(blocks, 1, 1);
+    launch(qer_prepare_q8, reinterpret_cast<const uint4*>(q), p.n_text, n_rows, h->n_pad, h->per_blk, p.n_heads,
+           p.n_kv_heads, p.head_dim, reinterpret_cast<uint4*>(h->d_qg));
   } else {
-    launch_dependent(true, qer_prepare_q, dim3(256), dim3(256), 0, st, q, p.n_text, n_rows, h->n_pad, h->per_blk, p.n_heads,
-                     p.n_kv_heads, p.head_dim, h->d_qg);
+    cfg.gridDim = dim3(256, 1, 1);
+    launch(qer_prepare_q, q, p.n_text, n_rows, h->n_pad, h->per_blk, p.n_heads, p.n_kv_heads, p.head_dim, h->d_qg);
   }
   const uint32_t grid = tiles < static_cast<uint32_t>(h->grid) ? tiles : static_cast<uint32_t>(h->grid);
   const uint32_t kk = static_cast<uint32_t>(std::max(1.0, std::nearbyint(static_cast<double>(p.rho) * n_frames)));
@@ -1271,22 +1301,6 @@ int cofie_qer_run(cofie_qer_t* h, const uint16_t* q, const uint16_t* k, uint32_t
       cudaEventRecord(e0, st);
     }
   }
-  // Every kernel may be scheduled while its predecessor still runs, and waits
-  // for it (griddepcontrol.wait) where it reads what that kernel or one before
-  // it wrote: every thread of the first kernel, which lets the scoring kernel
-  // start only after its wait, so that the keys are ready when that one does;
-  // the scoring kernel's q~ producer; every thread of the mean and ranking
-  // kernels. With the timing events in between, the scoring kernel's launch
-  // serialises as usual.
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  attr[1].id = cudaLaunchAttributeClusterDimension;
-  attr[1].val.clusterDim.x = 2;
-  attr[1].val.clusterDim.y = 1;
-  attr[1].val.clusterDim.z = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.stream = st;
   // One scoring pass per text block; passes after the first fold their
   // maxima into colmax (Eq. 7's max over all text tokens) and are ordered
   // after the pass before them as usual (no programmatic launch), so each
@@ -1304,22 +1318,20 @@ int cofie_qer_run(cofie_qer_t* h, const uint16_t* q, const uint16_t* k, uint32_t
       cfg.attrs = fold ? &attr[1] : attr;
       cfg.numAttrs = fold ? 1 : 2;
       const uint32_t n_chunks = h->D / kQerKChunk / h->pair_sub;
-      cudaLaunchKernelEx(&cfg, h->pair_sub == 2 ? qer_score_pair<2> : qer_score_pair<1>, map_k, map_q,
-                         static_cast<uint32_t>(nv), text_b, n_pad, fold, h->acc_cols, h->pair_key_slots,
-                         kQerPairQSlots, n_chunks, tiles, h->d_colmax, h->d_err, 2000000000ull);
+      launch(h->pair_sub == 2 ? qer_score_pair<2> : qer_score_pair<1>, map_k, map_q, static_cast<uint32_t>(nv), text_b, n_pad,
+             fold, h->acc_cols, h->pair_key_slots, kQerPairQSlots, n_chunks, tiles, h->d_colmax, h->d_err, 2000000000ull);
     } else {
       cfg.gridDim = dim3(grid, 1, 1);
       cfg.blockDim = dim3(kQerThreads, 1, 1);
       cfg.dynamicSmemBytes = h->smem;
       cfg.attrs = attr;
       cfg.numAttrs = fold ? 0 : 1;
-      cudaLaunchKernelEx(&cfg, qer_score, map_k, map_q, static_cast<uint32_t>(nv), text_b, n_pad, fold,
-                         h->acc_cols, h->n_buf, h->n_stages, h->D / kQerKChunk, tiles, h->d_colmax, h->d_err,
-                         2000000000ull);
+      launch(qer_score, map_k, map_q, static_cast<uint32_t>(nv), text_b, n_pad, fold, h->acc_cols, h->n_buf, h->n_stages,
+             h->D / kQerKChunk, tiles, h->d_colmax, h->d_err, 2000000000ull);
     }
   }
   if (e1) cudaEventRecord(e1, st);
-  if (!capturing) {
+  if (!capturing && e == cudaSuccess) {
     h->launches += 1;
     h->flops += 2.0 * h->n_blk * n_pad * static_cast<double>(nv) * h->D;
     h->key_bytes += 2.0 * static_cast<double>(nv) * h->D * h->n_blk;  // each pass reads the keys
@@ -1330,17 +1342,17 @@ int cofie_qer_run(cofie_qer_t* h, const uint16_t* q, const uint16_t* k, uint32_t
   if (n_frames <= kFewFrames) {
     cfg.gridDim = dim3(1, 1, 1);
     cfg.blockDim = dim3(kFewThreads, 1, 1);
-    cudaLaunchKernelEx(&cfg, qer_finish_few, static_cast<const float*>(h->d_colmax), n_frames, p.tokens_per_frame, scale, w,
-                       kk, sel_out, kdev);
+    launch(qer_finish_few, static_cast<const float*>(h->d_colmax), n_frames, p.tokens_per_frame, scale, w, kk, sel_out, kdev);
   } else {
     cfg.gridDim = dim3((n_frames + 7) / 8, 1, 1);
     cfg.blockDim = dim3(256, 1, 1);
-    cudaLaunchKernelEx(&cfg, qer_mean, static_cast<const float*>(h->d_colmax), n_frames, p.tokens_per_frame, scale, w);
+    launch(qer_mean, static_cast<const float*>(h->d_colmax), n_frames, p.tokens_per_frame, scale, w);
     cfg.gridDim = dim3((n_frames + kRankThreads / 32 - 1) / (kRankThreads / 32), 1, 1);
     cfg.blockDim = dim3(kRankThreads, 1, 1);
-    cudaLaunchKernelEx(&cfg, qer_rank, static_cast<const float*>(w), n_frames, kk, h->d_flag, h->d_done, sel_out, kdev);
+    launch(qer_rank, static_cast<const float*>(w), n_frames, kk, h->d_flag, h->d_done, sel_out, kdev);
   }
-  cudaError_t e = cudaGetLastError();
+  const cudaError_t last = cudaGetLastError();
+  if (e == cudaSuccess) e = last;
   if (e == cudaSuccess && kdev != k_out) {
     e = cudaStreamSynchronize(st);
     if (e == cudaSuccess) *k_out = *static_cast<volatile uint32_t*>(h->host_k);

@@ -338,3 +338,35 @@ def test_handles_of_different_text_lengths_alive_together(texts, d):
             w, s = f.run(q, k[: n * 256])
             assert torch.equal(w, w0) and torch.equal(s, s0)
         f.status()
+
+
+@pytest.mark.parametrize("n_frames", [20, 100])
+def test_a_launch_that_fails_ends_the_call(n_frames):
+    """A launch refused on the host (injected; nothing runs in its place): the
+    call says so and launches nothing after it, so that its outputs stay as
+    they were instead of holding what an earlier call left in the scratch."""
+    from paper_2609_03675_gb300 import QER, NGFFError, _abi
+    spec = S.QerSpec(n_text=300, n_heads=4, n_kv_heads=2, head_dim=64, n_frames=n_frames, tokens_per_frame=40, seed=5)
+    q, k, _ = S.generate(spec)
+    q, k = torch.from_numpy(q.view(np.int16)).cuda(), torch.from_numpy(k.view(np.int16)).cuda()
+    f = QER(spec.n_text, 4, 2, 64, n_frames, 40, 0.3)
+    w0, s0 = [x.clone() for x in f.run(q, k)]
+    hook = _abi.load().cofie_qer_debug_fail_launch
+    launches = 3 + (1 if n_frames <= 64 else 2)  # q~, two text blocks, the finishing kernels
+    try:
+        for after in range(launches):
+            w = torch.full((n_frames,), -7.0, device="cuda")
+            sel = torch.full((n_frames,), -7, dtype=torch.int32, device="cuda")
+            count = torch.full((1,), -7, dtype=torch.int32, device="cuda")
+            hook(after)
+            with pytest.raises(NGFFError) as e:
+                f.run_async(q, k, w, sel, count)
+            assert e.value.code == _abi.ECUDA
+            torch.cuda.synchronize()
+            assert bool((sel == -7).all()) and int(count) == -7
+            assert bool((w == -7).all()) or after == launches - 1 > 3  # the ranking follows the means
+    finally:
+        hook(-1)
+    w, s = f.run(q, k)
+    assert torch.equal(w, w0) and torch.equal(s, s0)
+    f.status()
