@@ -502,7 +502,7 @@ int run_segments(cofie_ngff* h, const SegTable& segs, cudaStream_t st, bool* kee
     if (e != cudaSuccess) return h->cuda_fail(e, "selection kernel launch");
     h->n_select += 1;
   } else {
-    e = launch_window(segs, sa, h->d_hist, h->d_ring, h->d_state, h->d_l1, h->d_mask, st, !ev0);
+    e = launch_window(segs, sa, h->d_hist, h->d_ring, h->d_state, h->d_l1, h->d_mask, h->num_sms, st, !ev0);
     if (e != cudaSuccess) return h->cuda_fail(e, "window kernel launch");
     e = launch_scan(segs, sa, h->d_l1, h->d_mask, h->d_hist, h->d_ring, h->d_state, st, !es0);
     if (e != cudaSuccess) return h->cuda_fail(e, "scan kernel launch");
@@ -1154,7 +1154,7 @@ int cofie_ngff_shard_prepare(cofie_ngff_t* h, uint32_t stream, const uint8_t* fr
   sh.s[0].stream = stream;
   sh.s[0].halo = n_halo;
   SelectArgs sa = select_args(h);
-  e = launch_window(sh, sa, h->d_hist, h->d_ring, h->d_state, h->d_l1, h->d_mask, st);
+  e = launch_window(sh, sa, h->d_hist, h->d_ring, h->d_state, h->d_l1, h->d_mask, h->num_sms, st);
   if (e == cudaSuccess) e = launch_gap_map(sh.s[0], sa, t0, h->d_mask, h->d_map, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(map_out, h->d_map, h->p.l_max * sizeof(uint16_t), cudaMemcpyDefault, st);
   if (e == cudaSuccess && classify(map_out) != kDevice) e = cudaStreamSynchronize(st);

@@ -394,8 +394,10 @@ cudaError_t launch_select_chain(const SegTable& segs, const SelectArgs& a, Chain
   const bool all = c.lags == a.l_max;
   const auto kernel = vec ? (all ? select_chain_kernel<true, true> : select_chain_kernel<true, false>)
                           : (all ? select_chain_kernel<false, true> : select_chain_kernel<false, false>);
-  const cudaError_t e = launch_dependent(pdl, kernel, dim3(c.n_tiles), dim3(kChainThreads), smem(c.lags), st, segs, a, c, hist,
-                                         ring, state);
+  const uint32_t sms = static_cast<uint32_t>(num_sms);
+  const size_t bytes = c.n_tiles <= sms ? spread_smem(smem(c.lags), c.n_tiles, sms) : smem(c.lags);
+  const cudaError_t e = launch_dependent(pdl, kernel, dim3(c.n_tiles), dim3(kChainThreads), bytes, st, segs, a, c, hist, ring,
+                                         state);
   return e == cudaSuccess ? cudaGetLastError() : e;
 }
 

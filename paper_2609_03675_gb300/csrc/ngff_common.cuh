@@ -98,6 +98,22 @@ inline cudaError_t launch_dependent(bool pdl, void (*kernel)(Params...), dim3 gr
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+// Shared memory for a programmatic dependent of `ctas` CTAs that takes `bytes`:
+// as much as lets an SM hold only its even share of them. Such CTAs are placed
+// while the kernel before still holds most SMs, and would otherwise crowd on
+// those that free first: four streams of 64 small frames, walked by a CTA each,
+// took 31.6 us a call from a graph with the four on one SM, 15.5 spread over
+// four; pushes of 400 frames of 1280x720 with the low-res signal, in 50 tiles
+// of 256-word rows, 216 us and 181. Up to three to an SM: more crowd little, and
+// 800 CTAs of distances (100 frames of each of 64 streams) took 4 us longer
+// spread. At most kSpreadSmem, the limit of kernels that are launched so.
+constexpr size_t kSpreadSmem = 115 * 1024;
+inline size_t spread_smem(size_t bytes, uint32_t ctas, uint32_t sms) {
+  const uint32_t share = (ctas + sms - 1) / sms;
+  const size_t least = 228u * 1024 / (share + 1) - 896;  // share + 1 CTAs, with 1 KiB each beside, are more than an SM has
+  return ctas > 1 && share <= 3 && bytes < least ? least : bytes;
+}
+
 // Index checks of the checked build (-DCOFIE_DEBUG_CHECKS=1), which stands in
 // for a memory checker: COFIE_BOUND(c) is true in normal builds (and
 // compiles away); in checked builds a false c sets this translation unit's
@@ -267,7 +283,8 @@ int hist_span_blocks_per_sm(int bin_path, uint32_t bins);
 cudaError_t launch_hist_span(const SegTable& segs, const HistArgs& a, const LumaConsts& lc, int bin_path, uint32_t* hist,
                              int grid, cudaStream_t st, bool pdl);
 cudaError_t launch_window(const SegTable& segs, const SelectArgs& a, const uint32_t* hist, const uint32_t* ring,
-                          const StreamState* state, uint32_t* l1, uint32_t* mask, cudaStream_t st, bool pdl = false);
+                          const StreamState* state, uint32_t* l1, uint32_t* mask, int num_sms, cudaStream_t st,
+                          bool pdl = false);
 cudaError_t launch_scan(const SegTable& segs, const SelectArgs& a, const uint32_t* l1, const uint32_t* mask,
                         uint32_t* hist, uint32_t* ring, StreamState* state, cudaStream_t st, bool pdl = false);
 uint32_t select_small_max();

@@ -52,6 +52,7 @@ constexpr uint32_t kPer = kLinkBlocks / kLinkWarps;  // blocks per warp
 constexpr uint32_t kScanFrames = kLinkThreads / 8;   // frames per pass of an open link's scan, four times as many
 constexpr uint32_t kScanNarrow = 64;                 // with rows of at most 64 words
 constexpr uint32_t kUnknown = 0xffffffffu;         // no keep among the staged rows, but frames beyond them
+static_assert((kStageWords + kMaxBins) * 4 <= kSpreadSmem, "the next kernel's limit");
 
 __device__ __forceinline__ uint32_t word_dist(uint32_t x, uint32_t y, uint32_t kind) {
   return kind == 1 ? static_cast<uint32_t>(__popc(x ^ y)) : (x > y ? x - y : y - x);
@@ -691,7 +692,7 @@ size_t lazy_scratch_words(uint32_t max_frames, uint32_t bins) {
 }
 
 cudaError_t lazy_prepare() {
-  const int walk = kLazyWalkSmem, next = (kStageWords + kMaxBins) * 4;
+  const int walk = kLazyWalkSmem, next = static_cast<int>(kSpreadSmem);
   cudaError_t e = cudaSuccess;
   const auto limit = [&](const auto k, int bytes) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
@@ -711,7 +712,8 @@ cudaError_t launch_lazy_walk(const SegTable& segs, const SelectArgs& a, uint32_t
   for (uint32_t i = 0; i < segs.count; ++i) longest = std::max(longest, segs.s[i].n);
   const bool vec = a.bins % 4 == 0 && a.dist_kind == 0;
   const cudaError_t e = launch_dependent(pdl, vec ? lazy_walk_kernel<true> : lazy_walk_kernel<false>, dim3(segs.count),
-                                         dim3(kLazyThreads), lazy_walk_smem(longest, a.bins, vec), st, segs, a, feat, ring, state);
+                                         dim3(kLazyThreads), spread_smem(lazy_walk_smem(longest, a.bins, vec), segs.count, kMaxSegs), st,
+                                         segs, a, feat, ring, state);
   return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
@@ -731,7 +733,8 @@ cudaError_t launch_lazy_select(const SegTable& segs, const SelectArgs& a, uint32
   uint32_t tiles = 0;
   for (uint32_t i = 0; i < segs.count; ++i) tiles += (segs.s[i].n + z.tile - 1) / z.tile;
   const bool vec = a.bins % 4 == 0 && a.dist_kind == 0;
-  const size_t smem = static_cast<size_t>(z.stage_rows + 1) * a.bins * 4;
+  const uint32_t sms = static_cast<uint32_t>(num_sms);
+  const size_t rows = static_cast<size_t>(z.stage_rows + 1) * a.bins * 4, smem = tiles <= sms ? spread_smem(rows, tiles, sms) : rows;
   cudaError_t e = launch_dependent(pdl, vec ? lazy_next_kernel<true> : lazy_next_kernel<false>, dim3(tiles),
                                    dim3(kLazyThreads), smem, st, segs, a, z, feat, static_cast<const uint32_t*>(ring),
                                    static_cast<const StreamState*>(state));

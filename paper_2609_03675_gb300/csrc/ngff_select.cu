@@ -651,7 +651,8 @@ cudaError_t launch_select_walk(const SegTable& segs, const SelectArgs& a, uint32
   const size_t smem = walk_smem_bytes(longest, a.l_max, a.mask_words, a.bins);
   const bool vec = a.bins % 4 == 0 && a.dist_kind == 0;
   const cudaError_t e = launch_dependent(pdl, vec ? select_walk_kernel<true> : select_walk_kernel<false>, dim3(segs.count),
-                                         dim3(kWalkThreads), smem, st, segs, a, hist, ring, state);
+                                         dim3(kWalkThreads), spread_smem(smem, segs.count, kMaxSegs), st, segs, a, hist, ring,
+                                         state);
   return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
@@ -681,6 +682,8 @@ cudaError_t scan_prepare() {
   const size_t scan = scan_smem_bytes(kMaxLmax / 32, kMaxLmax);
   limit(select_walk_kernel<true>, kWalkSmemMax);
   limit(select_walk_kernel<false>, kWalkSmemMax);
+  limit(window_kernel<true>, kSpreadSmem);
+  limit(window_kernel<false>, kSpreadSmem);
   limit(scan_kernel<false>, scan);
   limit(select_small_kernel<true, false>, scan);
   limit(select_small_kernel<false, false>, scan);
@@ -689,13 +692,14 @@ cudaError_t scan_prepare() {
 }
 
 cudaError_t launch_window(const SegTable& segs, const SelectArgs& a, const uint32_t* hist, const uint32_t* ring,
-                          const StreamState* state, uint32_t* l1, uint32_t* mask, cudaStream_t st, bool pdl) {
+                          const StreamState* state, uint32_t* l1, uint32_t* mask, int num_sms, cudaStream_t st, bool pdl) {
   const uint32_t grid = (segs.rows + kWinWarps - 1) / kWinWarps;
+  const size_t smem = pdl ? spread_smem(0, grid, static_cast<uint32_t>(num_sms)) : 0;
   const cudaError_t e =
       (a.bins % 4 == 0 && a.dist_kind == 0)
-          ? launch_dependent(pdl, window_kernel<true>, dim3(grid), dim3(kWinWarps * 32), 0, st, segs, a, hist, ring,
+          ? launch_dependent(pdl, window_kernel<true>, dim3(grid), dim3(kWinWarps * 32), smem, st, segs, a, hist, ring,
                              state, l1, mask)
-          : launch_dependent(pdl, window_kernel<false>, dim3(grid), dim3(kWinWarps * 32), 0, st, segs, a, hist, ring,
+          : launch_dependent(pdl, window_kernel<false>, dim3(grid), dim3(kWinWarps * 32), smem, st, segs, a, hist, ring,
                              state, l1, mask);
   return e == cudaSuccess ? cudaGetLastError() : e;
 }

@@ -97,3 +97,33 @@ def test_small_pushes_of_wide_rows(bins, l_max, scd):
     f.status()
     assert np.array_equal(torch.cat([k for _, k in got]).cpu().numpy(), ko)
     assert np.all(np.abs(torch.cat([s for s, _ in got]).cpu().numpy().astype(np.float64) - so) <= 1e-6 * so)
+
+
+def test_streams_of_a_batch_are_decided_side_by_side():
+    """A batched call of four streams runs one CTA per stream, on an SM each:
+    it takes little longer than the same call for one of them, not twice as
+    long (as when all four were placed on the first SM that came free)."""
+    from paper_2609_03675_gb300 import NGFF
+    n, us = 64, []
+    for S in (1, 4):
+        f = NGFF(64, 48, l_max=64, tau=0.15, max_streams=S)
+        fr = torch.randint(0, 256, (S, n, 48, 64, 3), dtype=torch.uint8, device="cuda")
+        out = [(torch.empty(n, device="cuda"), torch.empty(n, dtype=torch.uint8, device="cuda")) for _ in range(S)]
+        batch = f.make_batch([(s, fr[s], *out[s]) for s in range(S)])
+        f.push_batch_raw(*batch)
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            for _ in range(50):
+                f.push_batch_raw(*batch)
+        times = []
+        for _ in range(9):
+            a, b = torch.cuda.Event(True), torch.cuda.Event(True)
+            a.record()
+            g.replay()
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b))
+        f.status()
+        us.append(sorted(times)[4] * 20)
+    assert us[1] < 1.6 * us[0], us
