@@ -469,7 +469,7 @@ int run_segments(cofie_ngff* h, const SegTable& segs, cudaStream_t st, bool* kee
   // except where the window and scan kernels or the larger selection without
   // forced retention decide them: there one memset after the selection does
   const bool walk = select_walk_takes(longest, sa);
-  const bool chain = h->p.l_max > 0 && !walk && !sa.scd;
+  const bool chain = h->p.l_max > 0 && !walk && !sa.scd && select_chain_takes(segs, longest, sa, h->num_sms);
   const bool fused = longest <= select_small_max();
   const bool lazy_walk = h->p.l_max == 0 && lazy_walk_fits(longest, h->fw);
   if (*keep_hist && hist_out && (walk || chain || lazy_walk)) {

@@ -365,6 +365,28 @@ uint32_t chain_tile(const SegTable& segs, int num_sms) {
 
 }  // namespace
 
+// A tile's ticket, map and look-back are a fixed cost that pays where there are
+// distances to share out or a long scan to cut up. Left to the window and scan
+// kernels, of which the second takes a CTA per stream (us a push from a graph,
+// tiles / window and scan):
+//   one stream, at most 64 words of distances per frame (dHash with L_max up to
+//     32, histograms with L_max = 1), while 8-frame tiles are at most one per
+//     SM: 65 frames of 224x224, dHash, 13.4 / 12.0, 1000 of 64x48 22.9 / 19.6,
+//     but 4096 34.5 / 43.3; of histograms only past 500 frames (L_max = 1, 32
+//     bins: 130 frames 9.6 / 9.6, 1000 17.2 / 15.7);
+//   several streams and many frames, whose scans run beside one another: 70
+//     frames of each of 64 streams with 32 bins 38.4 / 32.5, 100 of 32 streams
+//     26.9 / 23.0, but 100 of 4 streams 10.5 / 11.2 and 300 of 64 streams 95.2 /
+//     106.5; with 256 bins and L_max = 1 140 of 32 streams 66.8 / 45.4, 100 of 8
+//     17.3 / 20.4.
+bool select_chain_takes(const SegTable& segs, uint32_t longest, const SelectArgs& a, int num_sms) {
+  if (longest <= select_small_max()) return true;
+  const uint32_t work = a.l_max * a.bins, rows = segs.rows;
+  if (segs.count == 1) return work > 64 || rows > 8u * num_sms || (a.dist_kind != 1 && rows < 500);
+  if (work <= 64) return rows < 500;
+  return work > 1024 || rows < (a.bins <= 64 ? 800u : 3000u) || rows > 9000;
+}
+
 uint32_t chain_max_tiles(uint32_t max_frames) { return max_frames / 8 + kMaxSegs + 1; }
 
 cudaError_t chain_prepare() {

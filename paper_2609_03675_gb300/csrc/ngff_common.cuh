@@ -296,7 +296,8 @@ cudaError_t launch_select_walk(const SegTable& segs, const SelectArgs& a, uint32
                                StreamState* state, cudaStream_t st, bool pdl = false);
 cudaError_t launch_cells_any(const SegTable& segs, const FeatArgs& fa, const LumaConsts& lc, uint32_t* cells,
                              int num_sms, cudaStream_t st, bool pdl = false);
-// pushes with L_max > 0 and no scene changes that are too large for the walk
+// whether tiles decide a push that is too large for the walk, or else the window and scan kernels
+bool select_chain_takes(const SegTable& segs, uint32_t longest, const SelectArgs& a, int num_sms);
 uint32_t chain_max_tiles(uint32_t max_frames);
 cudaError_t chain_prepare();
 cudaError_t launch_select_chain(const SegTable& segs, const SelectArgs& a, ChainArgs c, int num_sms, uint32_t* hist,

@@ -99,6 +99,37 @@ def test_small_pushes_of_wide_rows(bins, l_max, scd):
     assert np.all(np.abs(torch.cat([s for s, _ in got]).cpu().numpy().astype(np.float64) - so) <= 1e-6 * so)
 
 
+# Few distances per frame, or several streams: the window and scan kernels on
+# one side of a line, tiles on the other (500 and 8 x 152 frames of one stream,
+# 800, 3000 and 9000 of several, none of them short).
+@pytest.mark.parametrize("bins,l_max,calls", [
+    (32, 1, [(499,), (500,), (1216,), (1217,)]), (64, 1, [(500,)]), (65, 1, [(500,)]), (2, 32, [(1216,), (1217,)]),
+    (32, 30, [(66, 733), (67, 733), (300, 8700), (301, 8700)]), (32, 1, [(66, 433), (67, 433), (700, 9000)]),
+    (256, 2, [(99, 2900), (100, 2900), (65, 735)]), (32, 33, [(400, 500)])])
+def test_pushes_around_the_choice_of_kernel(bins, l_max, calls):
+    from paper_2609_03675_gb300 import NGFF
+    S, tau = len(calls[0]), 0.25
+    T = [sum(c[s] for c in calls) for s in range(S)]
+    fr = [_frames(T[s], seed=90 + s) for s in range(S)]
+    dev = [torch.from_numpy(x).cuda() for x in fr]
+    outs = [(torch.empty(t, dtype=torch.float32, device="cuda"), torch.empty(t, dtype=torch.uint8, device="cuda")) for t in T]
+    f = NGFF(W, H, bins=bins, l_max=l_max, tau=tau, max_streams=S, max_frames_per_push=10000)
+    at = [0] * S
+    for c in calls:
+        items = []
+        for s in range(S):
+            a, b = at[s], at[s] + c[s]
+            items.append((s, dev[s][a:b], outs[s][0][a:b], outs[s][1][a:b]))
+            at[s] = b
+        f.push_batch(items)
+    torch.cuda.synchronize()
+    f.status()
+    for s in range(S):
+        _, so, ko = oracle_run(fr[s], O.Params(W, H, bins=bins, l_max=l_max, tau=tau))
+        assert np.array_equal(outs[s][1].cpu().numpy(), ko), s
+        assert np.all(np.abs(outs[s][0].cpu().numpy().astype(np.float64) - so) <= 1e-6 * so), s
+
+
 def test_streams_of_a_batch_are_decided_side_by_side():
     """A batched call of four streams runs one CTA per stream, on an SM each:
     it takes little longer than the same call for one of them, not twice as
