@@ -38,6 +38,16 @@ def test_histograms_across_the_slice_sizes(w, h, frames, bins):
     f.status()
 
 
+@pytest.mark.parametrize("bins", [16, 64, 65, 128])
+@pytest.mark.parametrize("w,h,frames", [(640, 360, 69), (640, 360, 70), (3840, 2160, 2), (640, 360, 121), (640, 360, 122),
+                                        (160, 160, 626)])
+def test_histograms_around_the_even_shares(w, h, frames, bins):
+    """1,000,000 groups, from which launches of fewer than five long slices per
+    SM run in even shares, and 1,750,000, from which others do; frames too small
+    for shares; 64 bins, up to which they are used."""
+    test_histograms_across_the_slice_sizes(w, h, frames, bins)
+
+
 def test_more_rows_than_a_grid_dimension():
     from paper_2609_03675_gb300 import NGFF
     w, h, T = 16, 2, 70001
