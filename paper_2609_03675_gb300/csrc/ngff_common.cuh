@@ -309,7 +309,7 @@ cudaError_t launch_dhash_finish(uint32_t* cells, uint32_t rows, const FeatArgs& 
                                 bool pdl = false);
 cudaError_t launch_wait_probe(uint64_t timeout_ns, uint32_t* err, cudaStream_t st);
 // L_max = 0: pushes whose longest piece of a stream one CTA decides, and larger ones
-bool lazy_walk_fits(uint32_t longest, uint32_t bins);
+bool lazy_walk_fits(uint32_t longest, uint32_t streams, uint32_t bins);
 size_t lazy_scratch_words(uint32_t max_frames, uint32_t bins);
 cudaError_t lazy_prepare();
 cudaError_t launch_lazy_walk(const SegTable& segs, const SelectArgs& a, uint32_t* feat, uint32_t* ring, StreamState* state,

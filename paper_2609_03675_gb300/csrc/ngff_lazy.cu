@@ -4,8 +4,9 @@
 // stream's state between pushes is {t, the open scene-change run} and two ring
 // rows: slot 0 holds c_{t-1}, slot 1 holds c_{r(t)}.
 //
-// Pushes of at most kLazyWalkFrames frames per stream whose rows fit shared
-// memory (lazy_walk_kernel): one CTA per stream walks the rule in frame order.
+// Pushes of at most kLazyWalkFrames frames (more of each of several streams,
+// fewer of wide rows) whose rows fit shared memory (lazy_walk_kernel): one CTA
+// per stream walks the rule in frame order.
 //
 // Larger pushes, in three launches:
 //   lazy_next_kernel   which frame would follow frame r as a reference does
@@ -34,16 +35,24 @@
 namespace cofie {
 namespace {
 
-// One launch up to where the serial walk passes the cost of two more launches:
-// pushes of 130 frames of 224x224 took 31 us walked and 37 us linked, of 260
-// frames 42 (walked from global memory, without this limit) and 39 us.
-constexpr uint32_t kLazyWalkFrames = 192;
+// One launch up to where the serial walk passes the cost of two more. Which of
+// the two is faster depends on how often frames are kept, which the host does
+// not know (32 bins, us a push from a graph, walked / linked, with a keep every
+// 4, 20 and 300 frames): 260 frames 24.7 / 14.4, 11.4 / 14.5 and 10.0 / 20.6,
+// 400 35.7 / 15.6, 15.2 / 15.6 and 13.5 / 19.4, 500 45.5 / 16.0, 18.4 / 16.1 and
+// 16.0 / 20.1. The walks of several streams run beside one another: 16 streams
+// of 300 39.9 / 33.5, 24.0 / 33.8 and 22.2 / 56.2, 64 of 500 163.9 / 160.7, 136.8 /
+// 161.8 and 134.8 / 204.2.
+// With rows of more than 64 words a walk is slower and links are as fast (128
+// bins, 260 frames 56.6 / 19.3, 24.7 / 19.2 and 21.2 / 28.7).
+constexpr uint32_t kLazyWalkFrames = 384, kLazyWalkWideFrames = 256, kLazyWalkManyFrames = 512, kLazyMany = 4;
 constexpr size_t kLazyWalkSmem = 200 * 1024;
 constexpr uint32_t kWalkFew = 16;
 constexpr int kLazyThreads = 256;
 constexpr uint32_t kLazyWarps = kLazyThreads / 32;
 constexpr uint32_t kStageWords = 16384;  // 64 KiB of rows per CTA of the next kernel
 constexpr uint32_t kStageRows = 256;
+static_assert((kStageWords + kMaxBins) * 4 <= kSpreadSmem, "the next kernel's limit");
 constexpr int kLinkThreads = 1024;
 constexpr uint32_t kLinkWarps = kLinkThreads / 32;
 constexpr uint32_t kLinkBlocks = 128;              // blocks of 32 frames per pass of the chain kernel
@@ -52,7 +61,6 @@ constexpr uint32_t kPer = kLinkBlocks / kLinkWarps;  // blocks per warp
 constexpr uint32_t kScanFrames = kLinkThreads / 8;   // frames per pass of an open link's scan, four times as many
 constexpr uint32_t kScanNarrow = 64;                 // with rows of at most 64 words
 constexpr uint32_t kUnknown = 0xffffffffu;         // no keep among the staged rows, but frames beyond them
-static_assert((kStageWords + kMaxBins) * 4 <= kSpreadSmem, "the next kernel's limit");
 
 __device__ __forceinline__ uint32_t word_dist(uint32_t x, uint32_t y, uint32_t kind) {
   return kind == 1 ? static_cast<uint32_t>(__popc(x ^ y)) : (x > y ? x - y : y - x);
@@ -190,26 +198,27 @@ __global__ void __launch_bounds__(kLazyThreads) lazy_walk_kernel(SegTable segs, 
   }
   __syncthreads();
   if (warp == 0) {
-    // scene flags by twin comparison (one thread: their run is serial)
-    if (lane == 0) {
-      unsigned long long acc = acc0;
-      if (a.scd)
-        for (uint32_t j = 0; j < n; ++j) {
-          bool scene = false;
-          if (t0 + j != 0) {
-            const unsigned long long adj = sadj[j];
-            if (adj >= a.x_cut) {  // a cut ends the run
-              scene = true;
-              acc = 0;
-            } else if (adj >= a.x_grad) {  // joins the run: a gradual change where its sum first reaches T_b
-              acc += adj;
-              scene = acc >= a.x_cut && acc - adj < a.x_cut;
-            } else {  // a low difference ends the run
-              acc = 0;
-            }
-          }
-          scode[j] = scene;
+    // scene flags by twin comparison, 32 frames at a time: a cut (d_adj >= T_b)
+    // or a low difference (d_adj < T_s) ends the run, others join it, with a
+    // gradual change where its sum first reaches T_b
+    unsigned long long acc = acc0;
+    if (a.scd)
+      for (uint32_t f = 0; f < n; f += 32) {
+        const uint32_t j = f + lane;
+        const bool in = j < n && t0 + j != 0;
+        const unsigned long long adj = in ? sadj[j] : 0ull;
+        LzRun x = !in ? LzRun{0u, 0ull} : (adj >= a.x_cut || adj < a.x_grad) ? LzRun{1u, 0ull} : LzRun{0u, adj};
+#pragma unroll
+        for (uint32_t off = 1; off < 32; off <<= 1) {
+          if (off >= n) break;
+          const LzRun o = lz_shfl_up(x, off);
+          if (lane >= off) x = lz_cat(o, x);
         }
+        const unsigned long long run = x.reset ? x.sum : acc + x.sum;  // the run's sum at frame j
+        if (j < n) scode[j] = in && (adj >= a.x_cut || (adj >= a.x_grad && run >= a.x_cut && run - adj < a.x_cut));
+        acc = __shfl_sync(0xffffffffu, run, 31);
+      }
+    if (lane == 0) {
       state[sg.stream].t = t0 + n;
       state[sg.stream].g = 1;
       state[sg.stream].acc = acc;
@@ -682,8 +691,9 @@ constexpr size_t kLinkSmem = (2 * kLinkTile + 4 * kLinkBlocks) * 4;
 
 }  // namespace
 
-bool lazy_walk_fits(uint32_t longest, uint32_t bins) {
-  return longest <= kLazyWalkFrames && lazy_walk_smem(longest, bins, true) <= kLazyWalkSmem;
+bool lazy_walk_fits(uint32_t longest, uint32_t streams, uint32_t bins) {
+  const uint32_t most = streams >= kLazyMany ? kLazyWalkManyFrames : (bins > 64 ? kLazyWalkWideFrames : kLazyWalkFrames);
+  return longest <= most && lazy_walk_smem(longest, bins, true) <= kLazyWalkSmem;
 }
 
 // words of the larger pushes' scratch: adj, next, ref per frame, then next_pre, first and old_ref per segment

@@ -116,7 +116,7 @@ def test_batch_of_streams_without_gap():
         assert np.array_equal(torch.cat([k for _, k in outs[s]]).cpu().numpy(), ko), f"stream {s}"
 
 
-# Pushes on both sides of the single-kernel limit (192 frames, fewer with wide
+# Pushes on both sides of the single-kernel limit (384 frames, fewer with wide
 # rows) and of its ways to share out the pairs (16 frames), of the links'
 # tiles and staged rows (fewer with wide rows), and of the chain's passes of
 # 4096 frames; a still stream, whose links run past the staged rows, between
@@ -125,7 +125,7 @@ def test_batch_of_streams_without_gap():
                                             (64, 0.9, 0)])
 @pytest.mark.parametrize("scd", [False, True])
 @pytest.mark.parametrize("chunks", [[1, 16, 17, 7, 33, 2], [192, 193, 129, 64], [4096, 5], [3, 4097, 400],
-                                    [257, 1300, 66]])
+                                    [257, 1300, 66], [384, 385, 380]])
 def test_links_and_chain(chunks, bins, tau, still, scd):
     from paper_2609_03675_gb300 import NGFF, _abi
     w, h, T = 32, 8, sum(chunks)
@@ -155,7 +155,7 @@ def test_links_and_chain(chunks, bins, tau, still, scd):
 
 def test_batch_of_unequal_lengths_without_gap():
     from paper_2609_03675_gb300 import NGFF
-    calls = [(0, 1, 65, 700), (9, 70, 0, 8), (1, 64, 3, 2)]
+    calls = [(0, 1, 65, 700), (9, 70, 0, 8), (512, 64, 3, 2), (1, 513, 3, 2)]  # of four streams, 512 frames each are walked
     frs = [_frames(32, 8, sum(c[s] for c in calls), seed=790 + s, mean=6) for s in range(4)]
     f = NGFF(32, 8, tau=0.06, l_max=0, max_streams=4)
     dev = [torch.from_numpy(x).cuda() for x in frs]
