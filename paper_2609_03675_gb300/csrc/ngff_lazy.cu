@@ -210,13 +210,13 @@ __global__ void __launch_bounds__(kLazyThreads) lazy_walk_kernel(SegTable segs, 
         LzRun x = !in ? LzRun{0u, 0ull} : (adj >= a.x_cut || adj < a.x_grad) ? LzRun{1u, 0ull} : LzRun{0u, adj};
 #pragma unroll
         for (uint32_t off = 1; off < 32; off <<= 1) {
-          if (off >= n) break;
+          if (off >= n) break;  // lanes past the push are left out
           const LzRun o = lz_shfl_up(x, off);
           if (lane >= off) x = lz_cat(o, x);
         }
         const unsigned long long run = x.reset ? x.sum : acc + x.sum;  // the run's sum at frame j
         if (j < n) scode[j] = in && (adj >= a.x_cut || (adj >= a.x_grad && run >= a.x_cut && run - adj < a.x_cut));
-        acc = __shfl_sync(0xffffffffu, run, 31);
+        acc = __shfl_sync(0xffffffffu, run, min(n - f, 32u) - 1);
       }
     if (lane == 0) {
       state[sg.stream].t = t0 + n;
