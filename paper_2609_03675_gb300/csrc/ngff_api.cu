@@ -348,17 +348,18 @@ cudaError_t launch_first_stage(cofie_ngff* h, const SegTable& segs, cudaStream_t
   }
   // Which kernel, and the generic kernel's slices (16-pixel groups per CTA).
   // Launches of up to kGenericBins bins, and of frames that K1 does not take:
-  //  - fewer than five CTAs of kWaveGroups per SM and fewer than 1,000,000
-  //    groups: slices of 256 groups, as a programmatic dependent (pushes of 27
-  //    frames of 640x360 12.9 us on K1, 10.9; one 4K frame 10.8 on K1, 8.7; 60
-  //    frames 19.6 with kWaveGroups, 18.3); with many bins to clear and fold 512
-  //    from 480,000 groups on (40 frames, 128 bins: 21.3 on kWaveGroups, 20.5
-  //    with 256, 19.6 with 512);
+  //  - fewer than five CTAs of kWaveGroups per SM and, of aligned frames, fewer
+  //    than 1,000,000 groups: slices of 256 groups, as a programmatic dependent
+  //    (pushes of 27 frames of 640x360 12.9 us on K1, 10.9; one 4K frame 10.8 on
+  //    K1, 8.7; 60 frames 19.6 with kWaveGroups, 18.3); with many bins to clear
+  //    and fold 512 from 480,000 groups on (40 frames, 128 bins: 21.3 on
+  //    kWaveGroups, 20.5 with 256, 19.6 with 512; 16 unaligned frames of
+  //    1074x1132, 128 bins, 25.6 on kWaveGroups, 24.9 with 512);
   //  - up to one resident wave and an eighth of a second: aligned frames of at
   //    least kWaveGroups and up to 64 bins in even shares, where CTAs of
   //    kWaveGroups would be fewer than five per SM (two 4K frames 12.9 us, 16.2
   //    with 256 groups, 13.6 with kWaveGroups) and from 1,750,000 groups on
-  //    (serving calls of 133 frames of 640x360 20.7 us, 20 1080p frames from a
+  //    (serving calls of 133 frames of 640x360 21.7 us, 20 1080p frames from a
   //    graph 25.9 against 29.4; but 64 frames of 854x480, 64 bins, 29.0 against
   //    26.8); others in slices of kWaveGroups, as an ordinary launch, whose CTAs
   //    start as SMs free (the serving calls 24.1 us, 25.0 with half of that, 30.2
@@ -383,7 +384,7 @@ cudaError_t launch_first_stage(cofie_ngff* h, const SegTable& segs, cudaStream_t
     const uint64_t groups = static_cast<uint64_t>(h->npix / 16) * segs.rows;
     const uint32_t longer = h->lc.bins > 128 ? 2 : (h->lc.bins > 64 ? 1 : 0);
     const bool few = wave_ctas < 5 * sms;
-    if (few && groups < 1000000) return generic(longer && groups >= 480000 ? 512 : 256, pdl);
+    if (few && (!fast || groups < 1000000)) return generic(longer && groups >= 480000 ? 512 : 256, pdl);
     if (wave_ctas <= hi && fast && !longer && (few || groups >= 1750000) && ha.groups_per_frame >= kWaveGroups)
       return launch_hist_span(segs, ha, h->lc, h->bin_path, h->d_hist, h->span_grid, st, pdl);
     if (wave_ctas <= hi) return generic(kWaveGroups, false);
