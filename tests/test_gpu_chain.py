@@ -105,7 +105,8 @@ def test_small_pushes_of_wide_rows(bins, l_max, scd):
 @pytest.mark.parametrize("bins,l_max,calls", [
     (32, 1, [(499,), (500,), (1216,), (1217,)]), (64, 1, [(500,)]), (65, 1, [(500,)]), (2, 32, [(1216,), (1217,)]),
     (32, 30, [(66, 733), (67, 733), (300, 8700), (301, 8700)]), (32, 1, [(66, 433), (67, 433), (700, 9000)]),
-    (256, 2, [(99, 2900), (100, 2900), (65, 735)]), (32, 33, [(400, 500)])])
+    (256, 2, [(99, 2900), (100, 2900), (65, 735)]), (32, 33, [(400, 500)]),
+    (64, 30, [(200, 5000), (3, 5000)])])  # and a later stream of more tiles than one looks back on
 def test_pushes_around_the_choice_of_kernel(bins, l_max, calls):
     from paper_2609_03675_gb300 import NGFF
     S, tau = len(calls[0]), 0.25

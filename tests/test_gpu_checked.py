@@ -1,10 +1,11 @@
 """The checked build (kernels compiled with -DCOFIE_DEBUG_CHECKS=1, which
 check every computed index against their launch arguments and report a
 failed check through cofie_ngff_status) run over representative workloads:
-the fast and generic histogram kernels (odd sizes, an odd byte offset), the
-small-push walk kernel on staged and unstaged rows, one- and two-word gap masks, the
-spatial signals on both of their kernels, scene changes across scan tiles,
-the frame-order walk (L_max = 0), batches, shards, candidates and gather,
+the histogram kernels (slices of aligned and odd sizes, an odd byte offset, even
+shares, the bulk-copy ring), the small-push walk, the tiled selection with rows
+staged at once and in pieces, one- and two-word gap masks, the spatial signals on
+both of their kernels, scene changes across scan tiles and on wide rows, the walk
+and the links without forced retention, batches, shards, candidates and gather,
 and QER on both scoring kernels.
 Every result must still equal the oracle's and no check may fail. A memory
 checker is not available on the GPUs this is tested on; these checks stand in
@@ -59,7 +60,7 @@ def same(sg, kg, so, ko, label):
 
 
 n = 0
-# histogram: fast kernel (64x48) and generic kernel (37x23); L_max 7/30/40 (one and two mask words); B 32 and 7
+# histograms in slices, aligned (64x48) and not (37x23); L_max 7/30/40 (one and two mask words); B 32 and 7
 for (w, h) in ((64, 48), (37, 23)):
     fr = frames(w, h, 300, seed=600 + w)
     for bins, l_max in ((32, 30), (7, 7), (32, 40)):
@@ -70,8 +71,8 @@ for (w, h) in ((64, 48), (37, 23)):
             sg, kg = run(f, fr, chunks)
             same(sg, kg, so, ko, f"hist {w}x{h} B{bins} L{l_max} {chunks[:2]}")
             n += 1
-# frames at an odd byte offset (the generic kernel on a pixel count the fast kernel takes), and the
-# walk kernel reading 256-bin rows from global memory (too wide to stage) for pushes of 20 frames
+# frames at an odd byte offset, and 256-bin rows in pushes of 20 frames: too wide for the walk, in tiles
+# whose lags come in pieces (L_max = 256) or at once (64), or, with scene changes, walked all the same
 fr = frames(64, 48, 120, seed=690)
 raw = torch.empty(fr.nbytes + 64, dtype=torch.uint8, device="cuda")
 raw[3:3 + fr.nbytes].copy_(torch.from_numpy(fr.reshape(-1)))
@@ -80,19 +81,34 @@ f = NGFF(64, 48, tau=0.05, l_max=30)
 s1, k1 = f.push(raw[3:3 + fr.nbytes].view(fr.shape))
 torch.cuda.synchronize(); f.status()
 same(s1.cpu().numpy().astype(np.float64), k1.cpu().numpy(), so, ko, "generic kernel, offset 3"); n += 1
-_, so, ko = O.load().run(fr, O.Params(64, 48, bins=256, tau=0.05, l_max=64))
-f = NGFF(64, 48, bins=256, tau=0.05, l_max=64)
-same(*run(f, fr, [20] * 6), so, ko, "walk on unstaged 256-bin rows"); n += 1
-# spatial signals: streaming cell kernel (64x48) and per-frame kernel (72x40)
-for (w, h) in ((64, 48), (72, 40)):
-    fr = frames(w, h, 200, seed=640 + w)
+for l_max in (64, 256):
+    _, so, ko = O.load().run(fr, O.Params(64, 48, bins=256, tau=0.05, l_max=l_max))
+    f = NGFF(64, 48, bins=256, tau=0.05, l_max=l_max)
+    same(*run(f, fr, [20] * 6), so, ko, f"tiles of 256-bin rows, L_max {l_max}"); n += 1
+hist = np.stack([O.load().histogram(x, O.Params(64, 48, bins=256)) for x in fr])
+so, ko = SC.select(hist, O.Params(64, 48, bins=256, tau=0.3, l_max=64), 0.05, 0.01)
+f = NGFF(64, 48, bins=256, tau=0.3, l_max=64, signal=_abi.SIGNAL_SCD, scd_cut=0.05, scd_gradual=0.01)
+same(*run(f, fr, [20] * 6), so, ko, "scene changes on 256-bin rows"); n += 1
+# 256 bins on the bulk-copy kernel (fewer slices than two per SM), and even shares (over 1,000,000 groups)
+fr = frames(64, 48, 300, seed=691)
+_, so, ko = O.load().run(fr, O.Params(64, 48, bins=256, tau=0.05, l_max=30))
+f = NGFF(64, 48, bins=256, tau=0.05, l_max=30)
+same(*run(f, fr, [200, 100]), so, ko, "bulk-copy kernel, 256 bins"); n += 1
+fr = frames(640, 360, 75, seed=692)
+_, so, ko = O.load().run(fr, O.Params(640, 360, tau=0.05, l_max=30))
+f = NGFF(640, 360, tau=0.05, l_max=30)
+same(*run(f, fr, [75]), so, ko, "even shares"); n += 1
+# spatial signals: the ring (64x48 from 157 frames on, narrow cells; 640x360 from 18 on, wide ones) and slices
+# (the single frames; 72x40, whose width the ring does not take)
+for (w, h, T) in ((64, 48, 400), (72, 40, 200), (640, 360, 40)):
+    fr = frames(w, h, T, seed=640 + w)
     for kind in (SO.LOWRES, SO.DHASH):
         _, so, ko = SO.run(fr, O.Params(w, h, tau=0.05, l_max=11), kind)
         f = NGFF(w, h, tau=0.05, l_max=11, signal=kind)
-        sg, kg = run(f, fr, [100, 1, 99])
+        sg, kg = run(f, fr, [T // 2, 1, T // 2 - 1])
         same(sg, kg, so, ko, f"signal {kind} {w}x{h}")
         n += 1
-# scene changes over several 4096-frame scan tiles; and L_max = 0 (frame-order walk) for two signals
+# scene changes over several 4096-frame scan tiles; and L_max = 0 (walk and links) for two signals
 fr = frames(32, 24, 9000, seed=660, mean=40)
 hist = np.stack([O.load().histogram(x, O.Params(32, 24)) for x in fr])
 so, ko = SC.select(hist, O.Params(32, 24, tau=0.3, l_max=30), 0.05, 0.01)
@@ -191,4 +207,4 @@ def test_checked_build_runs_clean_and_matches_the_oracle():
                   build_dir=os.path.join(d, "obj"))
     r = subprocess.run([sys.executable, "-c", CHILD, lib, REPO], capture_output=True, text=True, timeout=900)
     assert r.returncode == 0, r.stdout[-2000:] + r.stderr[-4000:]
-    assert "checked workloads 27" in r.stdout, r.stdout[-2000:]
+    assert "checked workloads 33" in r.stdout, r.stdout[-2000:]

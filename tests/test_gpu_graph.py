@@ -4,8 +4,8 @@ A push with device frames and outputs may be enqueued while its CUDA stream
 captures a graph; every launch of the graph then decides the next frames of
 the stream. The decisions of a stream replayed that way, chunk by chunk
 from one input buffer, must be the oracle's single-pass result (Sec. 3.2,
-Eqs. 2-5), on every selection path (the fused small push, the windowed
-distances and scan of larger pushes, batches, L_max = 0) and with ordinary
+Eqs. 2-5), on the selection paths (the walk of small pushes, the tiles of larger
+ones, batches, the walk and the links without forced retention) and with ordinary
 pushes between the launches. Also the launch chaining those pushes rely on:
 frames written by a caller's kernel just before a push."""
 import numpy as np
@@ -44,7 +44,7 @@ def _capture(fn):
     return g
 
 
-@pytest.mark.parametrize("chunk", [8, 100])  # the fused small push; distances + scan + row clearing
+@pytest.mark.parametrize("chunk", [8, 100])  # the walk; tiles
 def test_captured_push_replays_the_stream(chunk):
     from paper_2609_03675_gb300 import NGFF
     T = 3 * chunk if chunk > 64 else 12 * chunk
@@ -140,9 +140,10 @@ def test_captured_batch_of_streams():
                torch.cat(got[s][1]).cpu().numpy())
 
 
-def test_captured_push_without_forced_retention():
+@pytest.mark.parametrize("chunk", [16, 400])  # walked; linked in three launches
+def test_captured_push_without_forced_retention(chunk):
     from paper_2609_03675_gb300 import NGFF
-    chunk, T = 16, 160
+    T = 160 if chunk < 160 else 3 * chunk
     spec, fr = _stream(T, seed=66)
     f = NGFF(spec.width, spec.height, tau=0.04, l_max=0)
     dev = torch.from_numpy(fr).cuda()
@@ -229,6 +230,35 @@ def test_frames_written_by_a_kernel_just_before_each_push(chunk):
     torch.cuda.synchronize()
     f.status()
     _check(fr, p, torch.cat(scores).cpu().numpy(), torch.cat(keep).cpu().numpy())
+
+
+@pytest.mark.parametrize("w,h,chunk,signal", [(640, 360, 75, "histogram"), (160, 91, 9, "lowres"), (161, 90, 9, "dhash")])
+def test_frames_written_just_before_pushes_that_fetch_ahead(w, h, chunk, signal):
+    """The same for the launches that have their frames fetched into the L2 cache
+    before they wait: even shares of a push of about one wave, and the sliced
+    cell sums of the spatial signals."""
+    from oracle import signals_oracle as SO
+    from paper_2609_03675_gb300 import NGFF, _abi
+    T = 4 * chunk
+    spec, fr = _stream(T, w=w, h=h, seed=70, mean=5)
+    kind = {"lowres": SO.LOWRES, "dhash": SO.DHASH}.get(signal)
+    f = NGFF(w, h, tau=0.05, l_max=9, signal={"lowres": _abi.SIGNAL_LOWRES, "dhash": _abi.SIGNAL_DHASH}.get(signal, 0))
+    gen = torch.Generator(device="cuda").manual_seed(6)
+    noise = torch.randint(0, 256, (chunk, h, w, 3), dtype=torch.uint8, device="cuda", generator=gen)
+    enc = [torch.bitwise_xor(torch.from_numpy(fr[i:i + chunk]).cuda(), noise) for i in range(0, T, chunk)]
+    buf = torch.empty_like(noise)
+    scores, keep = [], []
+    for e in enc:
+        torch.bitwise_xor(e, noise, out=buf)
+        s, k = f.push(buf)
+        scores.append(s)
+        keep.append(k)
+    torch.cuda.synchronize()
+    f.status()
+    p = O.Params(w, h, tau=0.05, l_max=9)
+    so, ko = SO.run(fr, p, kind)[1:] if kind else O.load().run(fr, p)[1:]
+    assert np.array_equal(torch.cat(keep).cpu().numpy(), ko)
+    assert np.all(np.abs(torch.cat(scores).cpu().numpy().astype(np.float64) - so) <= 1e-6 * so)
 
 
 @pytest.mark.parametrize("signal", ["lowres", "dhash"])

@@ -1,6 +1,7 @@
-"""L_max = 0 (no forced retention; Eq. 5's second term off): the rule walked
-in frame order by one warp per stream, against the oracles (C for the
-histogram, Python for the other signals) read the same way."""
+"""L_max = 0 (no forced retention; Eq. 5's second term off): the rule walked in
+frame order by one CTA per stream, or, in larger pushes, followed along links
+between reference frames, against the oracles (C for the histogram, Python for
+the other signals) read the same way."""
 import numpy as np
 import pytest
 import torch

@@ -1,8 +1,9 @@
 """Frames at the largest sizes the ABI accepts, where every 32-bit count,
 index and L1 numerator is closest to its limit: W·H just under 2^31 pixels
 (6.4 GB per frame; a histogram bin can hold every pixel and the L1 numerator
-2N stays below 2^32) on the fast kernel (W·H a multiple of 16) and on the
-generic one, and the low-res signal at its own limit of 2^24 pixels."""
+2N stays below 2^32) on the generic histogram kernel, aligned (W·H a multiple
+of 16) and not, and on the bulk-copy kernel (aligned, 256 bins), and the low-res
+signal at its own limit of 2^24 pixels."""
 import gc
 
 import numpy as np
@@ -45,20 +46,20 @@ def _limit_frames(w, h, seed):
     return fr.reshape(3, h, w, 3)
 
 
-@pytest.mark.parametrize("w,h", [(46336, 46336), (46339, 46342)])
-def test_histogram_at_the_pixel_limit(w, h):
+@pytest.mark.parametrize("w,h,bins", [(46336, 46336, 32), (46339, 46342, 32), (46336, 46336, 256)])
+def test_histogram_at_the_pixel_limit(w, h, bins):
     from paper_2609_03675_gb300 import NGFF
     assert w * h < 2**31 and 2 * w * h < 2**32
     T = 3
     fr = _limit_frames(w, h, seed=880 + (w * h) % 16)
-    p = O.Params(w, h, tau=0.02)
+    p = O.Params(w, h, bins=bins, tau=0.02)
     o = O.load()
     hist_o = o.histograms_parallel(fr.ctypes.data, T, p)
     so, ko = o.select(hist_o, p)
     dev = torch.from_numpy(fr).cuda()
     del fr
     gc.collect()
-    f = NGFF(w, h, tau=0.02, max_frames_per_push=T)
+    f = NGFF(w, h, bins=bins, tau=0.02, max_frames_per_push=T)
     s, k, hist = f.push(dev, return_hist=True)
     torch.cuda.synchronize()
     f.status()

@@ -1,10 +1,11 @@
-"""The first stage runs either the bulk-copy histogram kernel (K1) or the
-generic one, chosen per launch by its size: the generic kernel when its grid
-(one CTA per 2048 16-pixel groups of a frame) holds at least two CTAs per SM
-and fits one resident wave plus an eighth. Pushes sized just below, at and
-above those boundaries, plain and with histograms out, one stream and
-batched, give the oracle's histograms, scores and keep codes whichever
-kernel ran."""
+"""The first stage's kernel and slices are chosen per launch by its size. Up to
+128 bins the generic histogram kernel takes every launch, in short slices while
+long ones (2048 16-pixel groups of a frame) would be fewer than five CTAs per SM;
+with more bins it takes launches whose long slices are at least two CTAs per SM
+and fit one resident wave plus an eighth, and the bulk-copy kernel (K1) the
+others. Pushes sized just below, at and above those boundaries, plain and with
+histograms out, one stream and batched, give the oracle's histograms, scores
+and keep codes whichever kernel ran."""
 import numpy as np
 import pytest
 import torch
@@ -26,8 +27,8 @@ def n_sms():
 
 
 def _sizes(n):
-    # below and at 2 CTAs per SM; one wave at 6, 7 and 8 CTAs per SM; an eighth past 8; beyond
-    return [2 * n - 1, 2 * n, 6 * n, 7 * n, 8 * n, 9 * n, 9 * n + 1, 11 * n]
+    # below and at 2 and 5 CTAs per SM; one wave at 6, 7 and 8 CTAs per SM; an eighth past 8; beyond
+    return [2 * n - 1, 2 * n, 5 * n - 1, 5 * n, 5 * n + 1, 6 * n, 7 * n, 8 * n, 9 * n, 9 * n + 1, 11 * n]
 
 
 @pytest.mark.parametrize("bins,l_max,tau", [(32, 30, 0.05), (7, 33, 0.10), (256, 5, 0.02), (1, 1, 0.30)])
@@ -61,8 +62,8 @@ def test_pushes_across_the_first_stage_boundaries(n_sms, bins, l_max, tau):
 
 
 def test_batched_calls_across_the_boundaries(n_sms):
-    """Two streams per batched call whose combined frame count falls below,
-    inside and above the generic kernel's window."""
+    """Two streams per batched call whose combined frame count lies on both
+    sides of two and five CTAs per SM and of one wave and an eighth."""
     from paper_2609_03675_gb300 import NGFF
     per_call = [(n_sms - 1, n_sms - 1), (n_sms, n_sms), (3 * n_sms, 3 * n_sms), (4 * n_sms, 5 * n_sms),
                 (5 * n_sms, 5 * n_sms), (1, 2 * n_sms)]
@@ -92,15 +93,15 @@ def test_batched_calls_across_the_boundaries(n_sms):
     f.close()
 
 
-def test_bin_counts_around_the_ring_sizes():
-    """The bulk-copy kernel runs a shorter ring once the counters of many bins
-    would leave one CTA per SM: bin counts on both sides of that, on handles
-    alive together."""
+def test_bin_counts_on_both_histogram_kernels():
+    """Launches past one wave: the generic kernel up to 128 bins, the bulk-copy
+    kernel above, whose counters take more shared memory the more bins there
+    are, on handles alive together."""
     from paper_2609_03675_gb300 import NGFF
-    w, h, T = 1280, 720, 60  # past the generic kernel's window
+    w, h, T = 1280, 720, 60
     spec = synth.medium(seed=78).with_(width=w, height=h, frames=T, mean_scene_len=15)
     fr = synth.generate(spec)
     dev = torch.from_numpy(fr).cuda()
-    handles = {b: NGFF(w, h, bins=b, tau=0.05) for b in (256, 128, 127, 112, 64, 200)}
+    handles = {b: NGFF(w, h, bins=b, tau=0.05) for b in (256, 64, 128, 129, 200, 255)}
     for b, f in handles.items():
         assert_parity(run_stream(f, dev, [T]), oracle_run(fr, O.Params(w, h, bins=b, tau=0.05)), 0.05, f"B={b}")

@@ -81,7 +81,7 @@ def test_two_ramps_closed_form_on_device():
     from paper_2609_03675_gb300 import NGFF, _abi
     pos = [16 * t for t in range(21)] + [320] * 3 + [320 + 16 * (t - 23) for t in range(24, 64)]
     dev = torch.from_numpy(_frames_from_positions(pos)).cuda()
-    for l_max in (256, 0):  # the window + scan kernels, and the frame-order walk
+    for l_max in (256, 0):  # distances and scan in one kernel, and the walk without forced retention
         for chunks in ([64], [1] * 64, [5, 30, 29]):
             f = NGFF(W, H, tau=0.5, l_max=l_max, signal=_abi.SIGNAL_SCD, scd_cut=0.125, scd_gradual=0.01)
             _, k = _run(f, dev, chunks)
