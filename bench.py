@@ -613,7 +613,8 @@ def bench_gb300(args):
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                          "peak_kind": f"{peak_kind} copy bandwidth", "traffic": traffic,
                          "kernel": "ngff histogram (hist_generic_kernel)" if signal == 0
-                         else f"ngff {args.signal} cell sums (K1 cells)",
+                         else f"ngff {args.signal} cell sums "
+                              + ("(bulk-copy kernel)" if spec.width % 16 == 0 else "(cells_any_kernel)"),
                          "launch_ms": k1_ms, "bytes_per_launch": k1_bytes,
                          "select_ms_per_step": prof["select_ms"] / max(prof["select_timed"], 1)},
             "e2e": e2e,

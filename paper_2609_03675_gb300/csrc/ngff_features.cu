@@ -25,8 +25,10 @@ namespace {
 // 16 kAnyThreads pixels on, so its row and column advance by additions, and
 // its cell row by comparison with the row where the next one starts.
 //
-// Bound by memory latency: about 150 issue slots per 48 bytes, so the more
-// warps there are to cover a load, the nearer the kernel comes to DRAM's rate.
+// Bound by issue slots and load latency together: 208 instructions a warp for 32
+// groups of 48 bytes keep 64 % of the issue slots busy, DRAM runs at 68 % of its
+// peak, and over half of a warp's wait is for its loads, so the more warps there
+// are to cover them, the nearer the kernel comes to DRAM's rate.
 // Hence registers for six CTAs per SM and sums formed as the pixels are
 // decoded, without arrays of prefix sums (four CTAs: 5 % slower over 600
 // frames of 854x480; eight, which spill: 7 %). Lanes of a warp hold

@@ -233,7 +233,8 @@ __global__ void __launch_bounds__(kGatherThreads) gather_kernel(const uint8_t* _
 // two ends, are copied by bytes (fewer than 64 in all). Bound by DRAM as the
 // aligned copy is. It replaced a copy byte by byte, 265 us for 26 frames of
 // 1917x1080 (1.2 TB/s read and written); 300 such frames pushed, closed and
-// their candidates gathered went from 568 to 377 us.
+// their candidates gathered went from 568 to 377 us (365 with the other kernels of
+// now).
 template <bool kHostSrc>
 __global__ void __launch_bounds__(kGatherThreads) gather_any_kernel(const uint8_t* __restrict__ frames,
                                                                     uint32_t n_frames, uint64_t frame_bytes,

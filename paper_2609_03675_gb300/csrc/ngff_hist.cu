@@ -5,9 +5,11 @@
 // reading), bin = floor(Y B / 256), count[bin] += 1. Integer arithmetic only,
 // so the histogram is independent of summation order and bit-exact.
 //
-// Two kernels count them: the generic kernel below (any frame), which serves
-// histograms of up to 128 bins, and the fast kernel for more bins and for the
-// spatial signals, whose larger tables it clears and folds less often.
+// Three kernels count them: the generic kernel below (any frame), which serves
+// histograms of up to 128 bins in slices of frames; a variant of it that takes
+// launches of about one wave in even shares; and the fast kernel for more bins
+// and for the spatial signals, whose larger tables it clears and folds less
+// often.
 //
 // Fast kernel (frames of a multiple of 16 pixels, 16-byte aligned):
 //   - a persistent grid; each CTA owns a contiguous range of 24 KiB chunks of
@@ -462,8 +464,9 @@ __global__ void __launch_bounds__(kGenericThreads) hist_generic_kernel(SegTable 
 // leaves other SMs idle when slices of frames do so. While it waits a CTA has
 // the start of its share fetched into L2 (a hint; see the generic kernel):
 // kSpanAhead groups, 9 KiB, for all CTAs together 11 MB. Serving calls of 133
-// frames of 640x360 take 21.7 us against 24.1 in slices of 2048 groups; 22.4
-// with 64 groups ahead, 22.7 with 512, 25.6 with all of the share, 27 with none.
+// frames of 640x360 took 21.7 us (20.6 with the selection kernel of now) against
+// 24.1 in slices of 2048 groups; 22.4 with 64 groups ahead, 22.7 with 512, 25.6
+// with all of the share, 27 with none.
 constexpr uint32_t kSpanAhead = 192;
 
 template <int kBin>

@@ -14,9 +14,11 @@
 // that is kept: the text-by-vision score matrix is never written to memory,
 // which is the point of the paper's tiled computation.
 //
-// Kernels (one QER call launches four):
+// Kernels (one QER call launches the first, one of the scoring kernels per text
+// block, and the last one or the two before it):
 //   qer_prepare_q   q [n_text][H][d] -> q~ [N][D] bf16 (fp32 sums rounded to
-//                   nearest even; rows n_text..N-1 zero, N = n_text rounded up to 16)
+//                   nearest even; rows n_text..N-1 zero, N = n_text rounded up to
+//                   32, of which the one-SM kernel leaves out 16 that hold no text)
 //   qer_score       persistent CTAs over tiles of 256 visual tokens: TMA
 //                   (cp.async.bulk.tensor, 128-byte swizzle) streams 64-wide K
 //                   chunks of the token tile and of q~ into a shared-memory
@@ -31,11 +33,17 @@
 //   qer_mean        w_f = (sum of the frame's token maxima) / (|V_f| H sqrt(d)),
 //                   a warp per frame;
 //   qer_rank        the k best frames by rank (ties to the lower index), a
-//                   warp per frame; the last CTA writes them in time order.
+//                   warp per frame; the last CTA writes them in time order;
+//   qer_finish_few  both of them for up to 64 frames.
 // Every kernel is a programmatic dependent of the one before it (the first one
 // of the caller's, or of the call before), so its launch and set-up overlap
 // that kernel's tail; calls in a row take 2 us less each since the first
 // kernel is one too (128 frames of 40 text tokens 25.1 -> 23.4 us).
+// The scoring kernels load keys and write maxima without a wait of their own.
+// That is in order only because qer_prepare_q lets its dependents start after its
+// own wait: no scoring CTA exists before the kernel that wrote the keys, and the
+// call that last read the maxima, have completed. Signalled any earlier it
+// would be a race.
 // Every mbarrier wait is bounded by the global timer; a wait that runs out
 // sets an error bit, stops issuing, lets the work already issued finish
 // (bounded) and frees TMEM before the CTA exits.
